@@ -57,7 +57,7 @@
 // composite_batched_marked_kernel.
 #include <climits>
 
-#include "vdi_device.cuh"
+#include "vdi_search.cuh"
 
 namespace vdi {
 
@@ -321,6 +321,14 @@ __device__ __forceinline__ void mix_end(Mix& m, const RecC& c, float f, float b)
 }
 
 constexpr float kNoEvent = 3.0e38f;
+
+// list words 2 and 3: pieces taken from the pool (64 bits: what the lists ask for may exceed any pool)
+__device__ __forceinline__ unsigned long long* pool_used(uint32_t* list) {
+    return reinterpret_cast<unsigned long long*>(list + 2);
+}
+
+// slots of a pixel's run of n pieces in the pool (the search reads four pieces at once)
+__device__ __forceinline__ uint32_t run_slots(uint32_t n) { return (n + 3u) & ~3u; }
 
 // Heads in registers (K <= KMAX, fully unrolled; KMAX <= 8).
 template <int KMAX>
@@ -978,6 +986,45 @@ __global__ void __launch_bounds__(128, NLEV > 2 ? 2 : 3) composite_kernel(const 
 }
 
 
+// storage of the pieces of the pixels the lane and pooled staged paths search
+struct PiecePool {
+    float4* A;  // (P.rgb, a)
+    float2* B;  // (b, log2(1 - a))
+    uint32_t cap;
+};
+
+// list entry of a pixel for the flat search: pixel (top bit: composite it by the direct sweep), first
+// piece in the pool (a multiple of 4: four pieces are read at once), packed numbers of pieces, of non-transparent
+// pieces and of columns of its part of the pool (groups of four pieces lie that many groups apart), front of the
+// first piece
+struct FlatEntry {
+    uint32_t p, base, n_nt;
+    float f0;
+};
+
+// n and nt below 2048 (a stage of 1024 records has at most 2047 pieces, a lane's slab of 480 at most 959), 32 columns
+__device__ __forceinline__ uint32_t pieces_of(uint32_t n_nt) { return n_nt & 0x7FFu; }
+__device__ __forceinline__ uint32_t opaque_of(uint32_t n_nt) { return n_nt >> 11 & 0x7FFu; }
+__device__ __forceinline__ uint32_t columns_of(uint32_t n_nt) { return (n_nt >> 22) + 1u; }
+__device__ __forceinline__ uint32_t pack_pieces(uint32_t n, uint32_t nt, int ncol) {
+    return n | nt << 11 | (uint32_t)(ncol - 1) << 22;
+}
+
+// writes the zero tail, count and gamma of pixel p after an emission of `written` records
+__device__ __forceinline__ void finish_pixel(const OutDev& out, uint32_t p, int written, float gamma) {
+    for (int j = written; j < out.n_s; ++j) {
+        const size_t idx = (size_t)p * out.n_s + j;
+        if (out.prec == VDI_PREC_F32) {
+            reinterpret_cast<float4*>(out.rgba)[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
+            out.fb[idx] = make_float2(0.f, 0.f);
+        } else {
+            reinterpret_cast<uint4*>(out.rgba)[idx] = make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
+    out.counts[p] = (uint32_t)written;
+    if (out.gamma) out.gamma[p] = gamma;
+}
+
 // ---------------------------------------------------------------------------
 // Staged path
 // ---------------------------------------------------------------------------
@@ -993,19 +1040,44 @@ __global__ void __launch_bounds__(128, NLEV > 2 ? 2 : 3) composite_kernel(const 
 // bit for bit those of the direct sweep.  Pixels with more records than the
 // stage holds are listed for the direct path (a second launch).
 
-constexpr int kStageRMax = 1024;           // records per pixel held by the stage
-constexpr int kStageWarps = 8;             // warps per CTA
+// A pixel is built by one warp when its 32-pixel batch's lists are short, by a CTA of four when they are long:
+// the steps are chains of dependent shared-memory reads, so what counts is the warps an SM holds.  A warp's
+// stage of 1024 records (20 KB, a 172 KB CTA of 8 warps) left 8 warps per SM, 17% of the issue slots used; four
+// warps on such a stage make 40, and short lists take a stage of 320 records (7 KB) each.
+constexpr int kStageRMax = 1024;   // records per pixel held by the largest stage
+constexpr int kStageRSmall = 320;  // records per pixel of a batch that single warps build
+constexpr int kStageWarps = 4;     // warps per CTA, of either kind
 
+struct ScanState;
+
+template <int RMAX>
 struct StageSmem {
-    uint16_t pay[2][2 * kStageRMax];  // bounds: (valid record << 1) | is_back
-    float2 rfb[kStageRMax];           // bounds of the valid records
-    uint32_t rloc[kStageRMax];        // (PE << 16) | index in the PE's list, of the valid records
-    uint32_t pref[VDI_MAX_PE + 1];    // records before PE e
-    uint32_t vpref[VDI_MAX_PE + 1];   // valid records before PE e
-    uint64_t off[VDI_MAX_PE];         // start of PE e's list for the pixel
+    uint16_t pay[2][2 * RMAX];      // bounds: (valid record << 1) | is_back
+    float2 rfb[RMAX];               // bounds of the valid records
+    uint32_t rloc[RMAX];            // (PE << 16) | index in the PE's list, of the valid records
+    uint32_t pref[VDI_MAX_PE + 1];  // records before PE e
+    uint32_t vpref[VDI_MAX_PE + 1]; // valid records before PE e
+    uint64_t off[VDI_MAX_PE];       // start of PE e's list for the pixel
+    uint32_t nv, nt;
 };
 
-__device__ __forceinline__ float bound_key(const StageSmem& S, uint32_t w) {
+// NW warps working on one pixel: their threads' rank, barrier and vote
+template <int NW>
+__device__ __forceinline__ int group_rank() {
+    return NW == 1 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+}
+template <int NW>
+__device__ __forceinline__ void group_sync() {
+    if (NW == 1) __syncwarp();
+    else __syncthreads();
+}
+template <int NW>
+__device__ __forceinline__ bool group_any(bool v) {
+    return NW == 1 ? __any_sync(0xffffffffu, v) : __syncthreads_or(v) != 0;
+}
+
+template <int RMAX>
+__device__ __forceinline__ float bound_key(const StageSmem<RMAX>& S, uint32_t w) {
     const float2 fb = S.rfb[w >> 1];
     return (w & 1u) ? fb.y : fb.x;
 }
@@ -1073,8 +1145,8 @@ __device__ __forceinline__ ScanState shfl_up_state(const ScanState& v, int d) {
 }
 
 // applies bound w (sorted position i) to the state
-template <int PREC, bool OPQ>
-__device__ __forceinline__ void stage_apply(const PeIn* pe, const StageSmem& S, uint32_t w, ScanState& a) {
+template <int PREC, bool OPQ, int RMAX>
+__device__ __forceinline__ void stage_apply(const PeIn* pe, const StageSmem<RMAX>& S, uint32_t w, ScanState& a) {
     const uint32_t c = w >> 1;
     const uint32_t loc = S.rloc[c];
     const int e = (int)(loc >> 16);
@@ -1085,29 +1157,30 @@ __device__ __forceinline__ void stage_apply(const PeIn* pe, const StageSmem& S, 
     a.xr ^= c;
 }
 
-// Where phase G writes a pixel's pieces: a column of a warp's piece buffer
-// (rows 32 elements apart), or (POOL) a run of the pool allocated once the
-// pixel's piece count is known; base receives the run's first piece, and a
-// pixel whose run does not fit the pool gets npieces = -1 and no writes.
-struct PoolRun {
-    uint32_t* counter;
-    uint32_t cap;
-    uint32_t base;
+// Where phase G writes a pixel's pieces: column `col` of its batch's part of the pool, rows of 4 pieces by
+// `ncol` columns.  A lane of the search then reads whole sectors, and the lanes that search a batch's pixels
+// together read neighbouring ones.  (One run per pixel, allocated as it was built, put the runs of a batch 60 MB
+// apart: every lane of the search in pages of its own.)
+struct PoolColumn {
+    float4* A;  // of the batch's first piece
+    float2* B;
+    int col, ncol;
+    __device__ __forceinline__ size_t at(uint32_t row) const {
+        return ((size_t)(row >> 2) * ncol + col) * 4 + (row & 3);
+    }
 };
 
 // Phase G after the merge: exact prefix scan of the records' terms over the
 // sorted bounds (srt, E of them; nv valid records), in contiguous chunks per
-// lane, and the pieces written to the column (or the pool).
-template <int PREC, bool OPQ, bool POOL = false>
-__device__ __forceinline__ void stage_scan(const PeIn* pe, const StageSmem& S, const uint16_t* srt, uint32_t E,
-                                           uint32_t nv, float4* colA, float2* colB, int& npieces, int& nt,
-                                           float& f0, PoolRun* run = nullptr) {
-    constexpr size_t kStride = POOL ? 1 : 32;
-    const int lane = threadIdx.x & 31;
-    // exact prefix scan of the records' terms over the sorted bounds, in
-    // contiguous chunks per lane
-    const uint32_t chunk = (E + 31) / 32;
-    const uint32_t i0 = min(E, lane * chunk), i1 = min(E, i0 + chunk);
+// thread, and the pieces written to the column.  tot: scratch for the warps' totals.
+template <int NW, int PREC, bool OPQ, int RMAX>
+__device__ __forceinline__ void stage_scan(const PeIn* pe, StageSmem<RMAX>& S, ScanState* tot, const uint16_t* srt,
+                                           uint32_t E, uint32_t nv, const PoolColumn& out, int& npieces, int& nt,
+                                           float& f0) {
+    constexpr uint32_t T = 32 * NW;
+    const int lane = threadIdx.x & 31, rank = group_rank<NW>();
+    const uint32_t chunk = (E + T - 1) / T;
+    const uint32_t i0 = min(E, rank * chunk), i1 = min(E, i0 + chunk);
     ScanState loc;
     scan_reset(loc);
 #pragma unroll 4
@@ -1115,7 +1188,7 @@ __device__ __forceinline__ void stage_scan(const PeIn* pe, const StageSmem& S, c
         stage_apply<PREC, OPQ>(pe, S, srt[i], loc);
         if (i + 1 < E && bound_key(S, srt[i]) < bound_key(S, srt[i + 1])) ++loc.nb;
     }
-    // exclusive prefix of the lanes' totals
+    // exclusive prefix of the threads' totals
     ScanState inc = loc;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -1128,23 +1201,24 @@ __device__ __forceinline__ void stage_scan(const PeIn* pe, const StageSmem& S, c
     }
     ScanState st = shfl_up_state<OPQ>(inc, 1);
     if (lane == 0) scan_reset(st);
-    const uint32_t total_pieces = __shfl_sync(0xffffffffu, inc.nb, 31);
-    if constexpr (POOL) {
-        uint32_t base = 0;
-        if (lane == 0) base = atomicAdd(run->counter, total_pieces);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        run->base = base;
-        if ((uint64_t)base + total_pieces > (uint64_t)run->cap) {
-            npieces = -1;
-            nt = 0;
-            f0 = 0.f;
-            return;
+    uint32_t total_pieces;
+    if constexpr (NW == 1) {
+        total_pieces = __shfl_sync(0xffffffffu, inc.nb, 31);
+    } else {
+        if (lane == 31) tot[threadIdx.x >> 5] = inc;
+        __syncthreads();
+        total_pieces = 0;
+        for (int w = NW - 1; w >= 0; --w) {
+            total_pieces += tot[w].nb;
+            if (w < (int)(threadIdx.x >> 5)) {
+                ScanState t = tot[w];
+                scan_add<OPQ>(t, st);
+                st = t;
+            }
         }
-        colA += base;
-        colB += base;
     }
     // the pieces: after bound i the active set is that of [key_i, key_{i+1}]
-    int my_nt = 0;
+    uint32_t my_nt = 0;
     uint32_t row = st.nb;
     for (uint32_t i = i0; i < i1; ++i) {
         stage_apply<PREC, OPQ>(pe, S, srt[i], st);
@@ -1165,107 +1239,124 @@ __device__ __forceinline__ void stage_scan(const PeIn* pe, const StageSmem& S, c
         }
         Piece x;
         piece_from(st.s, whole, wc, t, t1, x);
-        colA[(size_t)row * kStride] = make_float4(x.P[0], x.P[1], x.P[2], x.a);
-        colB[(size_t)row * kStride] = make_float2(x.b, x.lgT);
+        const size_t at = out.at(row);
+        out.A[at] = make_float4(x.P[0], x.P[1], x.P[2], x.a);
+        out.B[at] = make_float2(x.b, x.lgT);
         my_nt += x.a > 0.f;
         ++row;
     }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) my_nt += __shfl_xor_sync(0xffffffffu, my_nt, d);
+    my_nt = __reduce_add_sync(0xffffffffu, my_nt);
     npieces = (int)total_pieces;
-    nt = my_nt;
     f0 = bound_key(S, srt[0]);
+    if constexpr (NW == 1) {
+        nt = (int)my_nt;
+    } else {
+        if (lane == 0) atomicAdd(&S.nt, my_nt);
+        __syncthreads();
+        nt = (int)S.nt;
+    }
 }
 
-// Phase G for pixel p into one column of the piece buffer (colA/colB point at
-// row 0 of the column; rows are 32 elements apart).  Returns false when the
-// pixel has more than kStageRMax records.
-template <int PREC, bool POOL = false>
-__device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem& S, float4* colA, float2* colB, int rows,
-                            int& npieces, int& nt, float& f0, PoolRun* run = nullptr) {
+// Phase G for pixel p (at most RMAX records) by NW warps.  Returns false when a list is out of depth order.
+template <int NW, int PREC, int RMAX>
+__device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem<RMAX>& S, ScanState* tot,
+                            const PoolColumn& out, int& npieces, int& nt, float& f0) {
+    constexpr uint32_t T = 32 * NW;
     const int lane = threadIdx.x & 31;
-    const unsigned lt_mask = (1u << lane) - 1u;
+    const uint32_t rank = (uint32_t)group_rank<NW>();
+    npieces = nt = 0;
+    f0 = 0.f;
     // counts and list starts, prefix over PEs
-    uint32_t c0 = 0, c1 = 0;
-    if (lane < k) {
-        c0 = __ldg(pe[lane].counts + p);
-        S.off[lane] = __ldg(pe[lane].offsets + p);
+    if (NW == 1 || threadIdx.x < 32) {
+        uint32_t c0 = 0, c1 = 0;
+        if (lane < k) {
+            c0 = __ldg(pe[lane].counts + p);
+            S.off[lane] = __ldg(pe[lane].offsets + p);
+        }
+        if (lane + 32 < k) {
+            c1 = __ldg(pe[lane + 32].counts + p);
+            S.off[lane + 32] = __ldg(pe[lane + 32].offsets + p);
+        }
+        const uint32_t x0 = warp_incl_scan_u32(c0);
+        const uint32_t t0 = __shfl_sync(0xffffffffu, x0, 31);
+        const uint32_t x1 = warp_incl_scan_u32(c1);
+        S.pref[lane] = x0 - c0;
+        S.pref[lane + 32] = t0 + x1 - c1;
+        if (lane == 31) S.pref[VDI_MAX_PE] = t0 + x1;
+        if (lane == 0) S.nt = 0;
     }
-    if (lane + 32 < k) {
-        c1 = __ldg(pe[lane + 32].counts + p);
-        S.off[lane + 32] = __ldg(pe[lane + 32].offsets + p);
+    group_sync<NW>();
+    const uint32_t R = S.pref[VDI_MAX_PE];
+    // every record's bounds, in list order
+    bool opaque = false, empty = false;
+    for (uint32_t r = rank; r < R; r += T) {
+        int lo = 0, hi = k - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (S.pref[mid] <= r) lo = mid;
+            else hi = mid - 1;
+        }
+        const uint32_t j = r - S.pref[lo];
+        float f, b;
+        load_fb<PREC>(pe[lo], S.off[lo] + j, f, b);
+        S.rfb[r] = make_float2(f, b);
+        S.rloc[r] = ((uint32_t)lo << 16) | j;
+        if (b > f) opaque |= rec_opaque(load_rec<PREC>(pe[lo], S.off[lo] + j));
+        else empty = true;
     }
-    const uint32_t x0 = warp_incl_scan_u32(c0);
-    const uint32_t t0 = __shfl_sync(0xffffffffu, x0, 31);
-    const uint32_t x1 = warp_incl_scan_u32(c1);
-    const uint32_t R = t0 + __shfl_sync(0xffffffffu, x1, 31);
-    S.pref[lane] = x0 - c0;
-    S.pref[lane + 32] = t0 + x1 - c1;
-    if (lane == 0) S.pref[VDI_MAX_PE] = R;
-    __syncwarp();
-    if (R > (uint32_t)kStageRMax) return false;
-    // bounds of every record; the valid ones (b > f) compacted in list order
-    uint32_t nv = 0;
-    bool opaque = false;
-    for (uint32_t r0 = 0; r0 < R; r0 += 32) {
-        const uint32_t r = r0 + lane;
-        bool valid = false;
-        float f = 0.f, b = 0.f;
-        int e = 0;
-        uint32_t j = 0;
-        if (r < R) {
-            int lo = 0, hi = k - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (S.pref[mid] <= r) lo = mid;
-                else hi = mid - 1;
+    uint32_t nv = R;
+    if (group_any<NW>(empty)) {
+        // drop the records with b <= f: the others move forward, in order
+        group_sync<NW>();
+        if (NW == 1 || threadIdx.x < 32) {
+            uint32_t n = 0;
+            for (uint32_t r0 = 0; r0 < R; r0 += 32) {
+                const uint32_t r = r0 + lane;
+                const float2 fb = r < R ? S.rfb[r] : make_float2(0.f, 0.f);
+                const uint32_t loc = r < R ? S.rloc[r] : 0u;
+                const bool valid = fb.y > fb.x;
+                const unsigned m = __ballot_sync(0xffffffffu, valid);
+                if (valid) {
+                    const uint32_t c = n + __popc(m & ((1u << lane) - 1u));
+                    S.rfb[c] = fb;
+                    S.rloc[c] = loc;
+                }
+                n += __popc(m);
+                __syncwarp();
             }
-            e = lo;
-            j = r - S.pref[e];
-            load_fb<PREC>(pe[e], S.off[e] + j, f, b);
-            valid = b > f;
-            if (valid) opaque |= rec_opaque(load_rec<PREC>(pe[e], S.off[e] + j));
+            if (lane == 0) S.nv = n;
         }
-        const unsigned m = __ballot_sync(0xffffffffu, valid);
-        if (valid) {
-            const uint32_t c = nv + __popc(m & lt_mask);
-            S.rfb[c] = make_float2(f, b);
-            S.rloc[c] = ((uint32_t)e << 16) | j;
+        group_sync<NW>();
+        nv = S.nv;
+        // valid records before PE e: the first compacted record of a PE >= e
+        for (int e = (int)rank; e <= k; e += (int)T) {
+            uint32_t lo = 0, hi = nv;
+            const uint32_t key = (uint32_t)e << 16;
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (S.rloc[mid] < key) lo = mid + 1;
+                else hi = mid;
+            }
+            S.vpref[e] = lo;
         }
-        nv += __popc(m);
+    } else {
+        for (int e = (int)rank; e <= k; e += (int)T) S.vpref[e] = e < k ? S.pref[e] : R;
     }
-    __syncwarp();
-    if (nv > 0 && 2 * nv - 1 > (uint32_t)rows) return false;  // more pieces than the column holds
+    group_sync<NW>();
     // each list must be in depth order (b of a record <= f of the next): else
     // the merge below would not be a permutation; such pixels go to the
     // direct path
     bool unsorted = false;
-    for (uint32_t c = lane + 1; c < nv; c += 32)
+    for (uint32_t c = rank + 1; c < nv; c += T)
         unsorted |= (S.rloc[c] >> 16) == (S.rloc[c - 1] >> 16) && !(S.rfb[c].x >= S.rfb[c - 1].y);
-    if (__any_sync(0xffffffffu, unsorted)) return false;
-    opaque = __any_sync(0xffffffffu, opaque);
-    // valid records before PE e: the first compacted record of a PE >= e
-    for (int e = lane; e <= k; e += 32) {
-        uint32_t lo = 0, hi = nv;
-        const uint32_t key = (uint32_t)e << 16;
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (S.rloc[mid] < key) lo = mid + 1;
-            else hi = mid;
-        }
-        S.vpref[e] = lo;
-    }
     const uint32_t E = 2 * nv;
-    for (uint32_t i = lane; i < E; i += 32) S.pay[0][i] = (uint16_t)i;
-    __syncwarp();
-    if (E == 0) {
-        npieces = 0;
-        nt = 0;
-        f0 = 0.f;
-        return true;
-    }
+    for (uint32_t i = rank; i < E; i += T) S.pay[0][i] = (uint16_t)i;
+    if (group_any<NW>(unsorted)) return false;
+    opaque = group_any<NW>(opaque);
+    group_sync<NW>();
+    if (E == 0) return true;
     // stable merge of the PEs' runs of bounds: round r merges the groups of
-    // 2^r PEs pairwise (merge path: every lane takes an equal share of the
+    // 2^r PEs pairwise (merge path: every thread takes an equal share of the
     // output, finds where it starts in the two runs by binary search and
     // merges sequentially from there; ties go to the lower run)
     int src = 0;
@@ -1274,8 +1365,8 @@ __device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem& S, flo
         uint16_t* outp = S.pay[src ^ 1];
         const int span = 2 << r;
         const int ngroups = (k + span - 1) / span;
-        const uint32_t per = (E + 31) / 32;
-        uint32_t o = min(E, (uint32_t)lane * per);
+        const uint32_t per = (E + T - 1) / T;
+        uint32_t o = min(E, rank * per);
         const uint32_t o_end = min(E, o + per);
         while (o < o_end) {
             // the merged group holding output o: the last one starting at or before o
@@ -1311,29 +1402,75 @@ __device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem& S, flo
             }
         }
         src ^= 1;
-        __syncwarp();
+        group_sync<NW>();
     }
     const uint16_t* srt = S.pay[src];
-    if (opaque) stage_scan<PREC, true, POOL>(pe, S, srt, E, nv, colA, colB, npieces, nt, f0, run);
-    else stage_scan<PREC, false, POOL>(pe, S, srt, E, nv, colA, colB, npieces, nt, f0, run);
-    __syncwarp();
+    if (opaque) stage_scan<NW, PREC, true>(pe, S, tot, srt, E, nv, out, npieces, nt, f0);
+    else stage_scan<NW, PREC, false>(pe, S, tot, srt, E, nv, out, npieces, nt, f0);
+    group_sync<NW>();
     return true;
 }
 
-
-// storage of the pieces of the pixels the lane and pooled staged paths search
-struct PiecePool {
-    float4* A;  // (P.rgb, a)
-    float2* B;  // (b, log2(1 - a))
-    uint32_t cap;
-};
-
-// list entry of a pixel for the flat search: pixel (top bit: composite it by the direct sweep), first
-// piece in the pool, number of pieces, front of the first piece
-struct FlatEntry {
-    uint32_t p, base, n;
+// One batch of 32 pixels (from p0 on, at most p1) of a request: if its longest pixel is this kernel's (more than
+// RMIN and at most RMAX records, or beyond every stage), allocates the batch's columns of the pool at once (its
+// longest pixel's bound for each) and builds them pixel by pixel.  emit(pixel, entry) is called by the lane of
+// warp 0 that has the pixel, for pixels with pieces and for those left to the direct sweep (the pixel's top bit);
+// pixels without records are finished here.
+struct BatchPixel {
+    bool have;
+    uint32_t p, base, n_nt;
     float f0;
 };
+
+template <int NW, int PREC, int RMIN, int RMAX>
+__device__ __forceinline__ bool build_batch(const PeIn* pe, int k, uint32_t p0, uint32_t p1, const OutDev& out,
+                                            const PiecePool& pool, unsigned long long* used,
+                                            StageSmem<RMAX>& S, ScanState* tot, unsigned long long* share, BatchPixel& mine) {
+    const int lane = threadIdx.x & 31;
+    const int ncol = (int)min(32u, p1 - p0);
+    // (every warp of the group sums the counts for itself)
+    uint32_t R = 0;
+    if (lane < ncol)
+        for (int e = 0; e < k; ++e) R += __ldg(pe[e].counts + p0 + lane);
+    const uint32_t fit = R <= (uint32_t)kStageRMax ? R : 0u;
+    const uint32_t longest = __reduce_max_sync(0xffffffffu, fit);
+    if (longest > (uint32_t)RMAX || (RMIN > 0 && longest <= (uint32_t)RMIN)) return false;
+    unsigned long long at = 0;
+    bool room = true;
+    if (longest > 0) {
+        const uint32_t need = run_slots(2 * longest - 1) * (uint32_t)ncol;
+        if (group_rank<NW>() == 0) at = atomicAdd(used, (unsigned long long)need);
+        if constexpr (NW == 1) {
+            at = __shfl_sync(0xffffffffu, at, 0);
+        } else {
+            if (threadIdx.x == 0) *share = at;
+            __syncthreads();
+            at = *share;
+        }
+        room = at + need <= (unsigned long long)pool.cap;
+    }
+    const uint32_t base = room ? (uint32_t)at : 0u;
+    mine.have = false;
+    for (int col = 0; col < ncol; ++col) {
+        const uint32_t p = p0 + (uint32_t)col;
+        const uint32_t n_rec = __shfl_sync(0xffffffffu, R, col);
+        int n = 0, nt = 0;
+        float f0 = 0.f;
+        bool ok = n_rec <= (uint32_t)kStageRMax && room;
+        if (ok && n_rec > 0)
+            ok = stage_pixel<NW, PREC>(pe, k, p, S, tot, PoolColumn{pool.A + base, pool.B + base, col, ncol}, n, nt, f0);
+        if (lane == col) {
+            if (!ok) {
+                mine = BatchPixel{true, p | 0x80000000u, 0u, 0u, 0.f};
+            } else if (n == 0) {
+                if (NW == 1 || threadIdx.x < 32) finish_pixel(out, p, 0, 0.f);  // no record: an empty list
+            } else {
+                mine = BatchPixel{true, p, base + (uint32_t)col * 4u, pack_pieces((uint32_t)n, (uint32_t)nt, ncol), f0};
+            }
+        }
+    }
+    return true;
+}
 
 // ---------------------------------------------------------------------------
 // Lane-staged path (short lists: K <= kLaneKMax).  Two passes.
@@ -1704,22 +1841,7 @@ struct LaneSink {
     }
 };
 
-// writes the zero tail, count and gamma of pixel p after an emission of `written` records
-__device__ __forceinline__ void finish_pixel(const OutDev& out, uint32_t p, int written, float gamma) {
-    for (int j = written; j < out.n_s; ++j) {
-        const size_t idx = (size_t)p * out.n_s + j;
-        if (out.prec == VDI_PREC_F32) {
-            reinterpret_cast<float4*>(out.rgba)[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
-            out.fb[idx] = make_float2(0.f, 0.f);
-        } else {
-            reinterpret_cast<uint4*>(out.rgba)[idx] = make_uint4(0u, 0u, 0u, 0u);
-        }
-    }
-    out.counts[p] = (uint32_t)written;
-    if (out.gamma) out.gamma[p] = gamma;
-}
-
-// list: [0] entries, [1] next entry for the search pass, [2] pieces taken from the pool, [3] unused,
+// list: [0] entries, [1] next entry for the search pass, [2], [3] pieces taken from the pool,
 // then FlatEntry entries from word 4
 struct LaneArgs {
     unsigned int* counter;  // batch counter of the batch pass
@@ -1882,14 +2004,15 @@ __global__ void __launch_bounds__(kLaneWarps * 32) composite_lane_kernel(const _
                 search = !emit;
             }
             // the searching lanes' pool runs (one atomic per warp)
-            uint32_t base = 0;
+            unsigned long long base = 0;
             bool fits = false;
             if (__any_sync(0xffffffffu, search)) {
-                const uint32_t mine = search ? bound : 0u;
+                const uint32_t mine = search ? run_slots(bound) : 0u;
                 const uint32_t inc = warp_incl_scan_u32(mine);
-                if (lane == 31) base = atomicAdd(la.list + 2, inc);
+                if (lane == 31) base = atomicAdd(pool_used(la.list), (unsigned long long)inc);
                 base = __shfl_sync(0xffffffffu, base, 31) + inc - mine;
-                fits = search && (uint64_t)base + mine <= (uint64_t)la.pool.cap;
+                fits = search && base + mine <= (unsigned long long)la.pool.cap;
+                if (!fits) base = 0;
             }
             // one sweep: the gamma = 0 pixels' records, the searched pixels' pieces
             LaneSink snk{&a.out, (size_t)p * a.out.n_s, 0, emit, la.pool.A + base, la.pool.B + base, fits, 0.f, 0u};
@@ -1906,7 +2029,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32) composite_lane_kernel(const _
                 }
             }
             if (__any_sync(0xffffffffu, search))
-                list_push(la.list, search, FlatEntry{fits ? p : (p | 0x80000000u), base, snk.np, snk.f0});
+                list_push(la.list, search, FlatEntry{fits ? p : (p | 0x80000000u), (uint32_t)base, pack_pieces(snk.np, (uint32_t)nt, 1), snk.f0});
             __syncwarp();
         }
     }
@@ -1929,111 +2052,136 @@ struct BuildArgs {
     uint32_t p0, p1;        // the chunk's pixels
 };
 
-template <int PREC, bool CENSUS>
-__global__ void __launch_bounds__(kStageWarps * 32, 1) composite_build_kernel(const __grid_constant__ CompArgs a,
-                                                                              const __grid_constant__ BuildArgs ba) {
-    extern __shared__ __align__(16) unsigned char stage_smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    StageSmem& S = reinterpret_cast<StageSmem*>(stage_smem)[warp];
+// shared memory of a build CTA: four warps' stages, or one stage for four warps
+template <int NW, int RMAX>
+struct BuildShared {
+    StageSmem<RMAX> stage[NW == 1 ? kStageWarps : 1];
+    ScanState tot[NW == 1 ? 1 : NW];
+    unsigned long long base;
+    uint32_t item;
+    __device__ BuildShared() {}
+};
+
+// the next item for a warp (NW = 1) or the CTA
+template <int NW>
+__device__ __forceinline__ uint32_t next_item(unsigned int* counter, uint32_t* share) {
+    uint32_t item = 0;
+    if (group_rank<NW>() == 0) item = atomicAdd(counter, 1u);
+    if constexpr (NW == 1) return __shfl_sync(0xffffffffu, item, 0);
+    __syncthreads();
+    if (threadIdx.x == 0) *share = item;
+    __syncthreads();
+    return *share;
+}
+
+template <int NW, int PREC, bool CENSUS>
+__global__ void __launch_bounds__(kStageWarps * 32) composite_build_kernel(const __grid_constant__ CompArgs a,
+                                                                          const __grid_constant__ BuildArgs ba) {
+    constexpr int RMAX = NW == 1 ? kStageRSmall : kStageRMax, RMIN = NW == 1 ? 0 : kStageRSmall;
+    __shared__ BuildShared<NW, RMAX> sh;
     const uint32_t nbatch = (ba.p1 - ba.p0 + 31u) / 32u;
     CompCensus cs;
     while (true) {
-        uint32_t batch = 0;
-        if (lane == 0) batch = atomicAdd(ba.counter, 1u);
-        batch = __shfl_sync(0xffffffffu, batch, 0);
+        const uint32_t batch = next_item<NW>(ba.counter + (NW == 1 ? 0 : 1), &sh.item);
         if (batch >= nbatch) break;
-        const uint32_t base = ba.p0 + batch * 32u;
-        FlatEntry mine{0u, 0u, 0u, 0.f};
-        bool have = false;
-        for (int col = 0; col < 32; ++col) {
-            const uint32_t p = base + (uint32_t)col;
-            if (p >= ba.p1) break;
-            PoolRun run{ba.list + 2, ba.pool.cap, 0u};
-            int n = 0, nt = 0;
-            float f0 = 0.f;
-            const bool ok = stage_pixel<PREC, true>(a.pe, a.k, p, S, ba.pool.A, ba.pool.B, 0x7FFFFFFF, n, nt, f0, &run);
-            if (lane == col) {
-                if (!ok || n < 0) {
-                    mine = FlatEntry{p | 0x80000000u, 0u, 0u, 0.f};
-                    have = true;
-                } else if (n == 0) {
-                    finish_pixel(a.out, p, 0, 0.f);  // no record: an empty list
-                    if (CENSUS) cs.pixels += 1;
-                } else {
-                    mine = FlatEntry{p, run.base, (uint32_t)n, f0};
-                    have = true;
-                }
-            }
+        BatchPixel px;
+        if (!build_batch<NW, PREC, RMIN, RMAX>(a.pe, a.k, ba.p0 + batch * 32u, ba.p1, a.out, ba.pool, pool_used(ba.list),
+                                               sh.stage[NW == 1 ? threadIdx.x >> 5 : 0], sh.tot, &sh.base, px))
+            continue;
+        if (NW > 1 && threadIdx.x >= 32) continue;
+        list_push(ba.list, px.have, FlatEntry{px.p, px.base, px.n_nt, px.f0});
+        if (CENSUS) {
+            const uint32_t p = ba.p0 + batch * 32u + (threadIdx.x & 31);
+            cs.pixels += !px.have && p < ba.p1;
         }
-        list_push(ba.list, have, mine);
     }
     if (CENSUS) census_flush(cs, reinterpret_cast<WsHeader*>(a.status)->counters);
 }
 
 // ---------------------------------------------------------------------------
-// Flat search: composite_search_emit<2> for one pixel per lane, written as one
-// loop whose body handles one piece of the lane's current march.  Lanes at
+// Flat search: the search and the emission of one pixel per lane, written as one
+// loop whose body handles four pieces of the lane's current march.  Lanes at
 // different marches, or at different pixels, execute the same loop body, so
 // a warp's lanes stay busy however many marches their pixels need; a lane
-// that finishes its pixel takes the next one from the list.  The decisions,
-// the table of decision intervals and the replay of sequential bisection are
-// those of composite_search_emit, step for step, so the output is the same,
-// bit for bit.  The pieces come from a pool in the workspace (written by the
-// batch pass), one contiguous run per pixel.
+// that finishes its pixel takes the next one from the list.  The decisions
+// are those of composite_search_emit, step for step, and the bisection is
+// replayed from the marches' counts (vdi_search.cuh), so the output is the
+// same, bit for bit.  The pieces come from a pool in the workspace (written by
+// the batch pass), one contiguous run per pixel.
+//
+// What bounds it: instructions per piece.  Four candidates run as two packed
+// pairs in the form that takes the fewest operations:
+//   - a closed S is P = A = L2 = 0, and the next non-transparent piece opens a new
+//     one;
+//   - opening is absorbing into the zeroed state (T = 1 - 0, fma(1, x, 0) = x):
+//     the state is multiplied by 0 or 1 instead of selected value by value, and
+//     a transparent piece that terminates S leaves the closed state;
+//   - the pieces are contiguous, so S's back is the next piece's front;
+//   - nA = -A saves the negations, products and sums keeping their bits;
+//   - an opaque piece's log2(1 - a) = -inf becomes -1e34, whose products with a
+//     length ratio give 2^x = 0 as well and which 0 clears.
+// The rounded operations that decide are cq_step's, in its order.
 // ---------------------------------------------------------------------------
-enum : int { kFlatIdle = 0, kFlatFirst = 1, kFlatSearch = 2, kFlatEmit = 3 };
-
 #ifndef VDI_FLAT_END_BATCH
 #define VDI_FLAT_END_BATCH 16
 #endif
 // resident CTAs of the flat pass per SM over the dense pieces of the pooled and batched paths (the lane
-// path takes as many as the registers allow): with 2047-piece runs, more lanes per SM evict each
-// other's pool lines and decision tables from L1 (dense 512^2, K = 32: 137.7 ms at 5 CTAs, 150.8 at 6;
-// the plain frame: 3.20 ms at 6, 3.36 at 5)
+// path takes as many as the registers allow)
 #ifndef VDI_FLAT_CTAS_PER_SM
 #define VDI_FLAT_CTAS_PER_SM 5
 #endif
 
-struct FlatLane {
-    const OutDev* out;  // the pixel's output (its request's, in a batch)
-    uint32_t p, base, n, j;
-    float f, f0;
-    int phase;
-    float g2[3];
-    CompCountQ st[3];  // a counting march's candidates; st[0] also holds the emission's supersegment
-    int nt;
-    float bt;  // emission: back of the last non-transparent piece of the open supersegment
-    int written;
-    float lo, hi, gamma;
-    int cnt_hi, it, count;
+#ifndef VDI_FLAT_MIN_BLOCKS
+#define VDI_FLAT_MIN_BLOCKS 5
+#endif
+
+struct FlatPair {
+    f32x2 P[3], nA, L2, f, kept;  // kept: non-transparent pieces absorbed (the others each opened an S)
 };
 
-__device__ __forceinline__ void flat_start_count(FlatLane& L, float lo, float hi) {
-    float g[3];
-    tree_candidates<2>(lo, hi, g);
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        L.g2[q] = __fmul_rn(g[q], g[q]);
-        L.st[q].cnt = 0;
-        L.st[q].open = false;
-        L.st[q].qlo = -1.f;
-        L.st[q].qhi = 3.0e38f;
-    }
-    L.nt = 0;
-    L.j = 0;
-    L.f = L.f0;
+// the closed state before a first piece with front f0 (any front of S before f0 will do)
+__device__ __forceinline__ void fp_reset(FlatPair& s, float f0) {
+    s.P[0] = s.P[1] = s.P[2] = s.nA = s.L2 = s.kept = pk(0.f);
+    s.f = pk(f0 - fmaxf(fabsf(f0), 1.f));
 }
 
-__device__ __forceinline__ void flat_start_emit(FlatLane& L) {
-    L.phase = kFlatEmit;
-    L.g2[0] = __fmul_rn(L.gamma, L.gamma);
-    L.st[0].cnt = 0;
-    L.st[0].open = false;
-    L.bt = 0.f;
-    L.written = 0;
-    L.j = 0;
-    L.f = L.f0;
+// A piece's values, each in both halves
+struct PieceX {
+    f32x2 P[3], na, lgT, f, lx, nt;
+};
+
+// where S goes on (1), or is closed or terminated by the piece (0); `last`: the first candidate's S is never terminated
+__device__ __forceinline__ f32x2 fp_keep(const FlatPair& s, const PieceX& x, f32x2 g2, bool last) {
+    float l0, l1, t0, t1, d0, d1, a0, a1;
+    unpk(fma2(s.f, pk(-1.f), x.f), l0, l1);
+    unpk(mul2(s.L2, mul2(x.lx, pk(rcp_approx(l0), rcp_approx(l1)))), t0, t1);
+    const f32x2 at = fma2(pk(ex2_approx(t0), ex2_approx(t1)), pk(-1.f), pk(1.f));
+    const f32x2 e0 = fma2(s.P[0], at, mul2(s.nA, x.P[0]));
+    const f32x2 e1 = fma2(s.P[1], at, mul2(s.nA, x.P[1]));
+    const f32x2 e2 = fma2(s.P[2], at, mul2(s.nA, x.P[2]));
+    unpk(fma2(e2, e2, fma2(e1, e1, mul2(e0, e0))), d0, d1);
+    unpk(mul2(g2, mul2(s.nA, s.nA)), t0, t1);
+    unpk(s.nA, a0, a1);
+    return pk(a0 == 0.f || (d0 >= t0 && !last) ? 0.f : 1.f, a1 == 0.f || d1 >= t1 ? 0.f : 1.f);
 }
+
+__device__ __forceinline__ void fp_apply(FlatPair& s, const PieceX& x, f32x2 k) {
+    const f32x2 A = mul2(s.nA, k);
+    const f32x2 T = add2(A, pk(1.f));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) s.P[c] = fma2(T, x.P[c], mul2(s.P[c], k));
+    s.nA = fma2(T, x.na, A);
+    s.L2 = add2(mul2(s.L2, k), x.lgT);
+    s.f = fma2(s.f, k, mul2(x.f, fma2(k, pk(-1.f), pk(1.f))));
+    s.kept = fma2(k, x.nt, s.kept);
+}
+
+struct FlatLane {
+    const OutDev* out;  // the pixel's output (its request's, in a batch)
+    uint32_t p, base;
+    int n, nt, ncol;
+    float f0;
+};
 
 __device__ __forceinline__ void flat_store(const OutDev& out, uint32_t p, int written, float f, float b,
                                            const float P[3], float A, float L2) {
@@ -2046,83 +2194,21 @@ __device__ __forceinline__ void flat_store(const OutDev& out, uint32_t p, int wr
     }
 }
 
-// Continues the bisection replay from level L.it: levels whose midpoint a recorded decision interval
-// answers need no march; returns with the next march started, or with the emission started.
-template <bool CENSUS>
-__device__ __forceinline__ void flat_advance(FlatLane& L, CountTable& t, int iters, int n_s, CompCensus& cs) {
-    while (L.it < iters) {
-        const float mid = 0.5f * (L.lo + L.hi);
-        const int c = t.lookup(__fmul_rn(mid, mid));
-        if (c < 0) {
-            L.phase = kFlatSearch;
-            flat_start_count(L, L.lo, L.hi);
-            return;
-        }
-        if (CENSUS) cs.table_hits += 1;
-        ++L.it;
-        if (c <= n_s) {
-            L.hi = mid;
-            L.cnt_hi = c;
-            if (c == n_s) break;
-        } else {
-            L.lo = mid;
-        }
-    }
-    L.gamma = L.hi;
-    L.count = L.cnt_hi;
-    flat_start_emit(L);
+// the first candidate's open supersegment as a record that ends at bt
+__device__ __forceinline__ void flat_record(const FlatLane& L, const FlatPair& s, int written, float bt) {
+    float P[3], nA, L2, f, u;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) unpk(s.P[c], P[c], u);
+    unpk(s.nA, nA, u);
+    unpk(s.L2, L2, u);
+    unpk(s.f, f, u);
+    flat_store(*L.out, L.p, written, f, bt, P, -nA, L2);
 }
 
-template <bool CENSUS>
-__device__ __forceinline__ void flat_end_march(FlatLane& L, CountTable& t, const OutDev& out, int iters,
-                                               unsigned int* status, CompCensus& cs) {
-    if (CENSUS) {
-        cs.sweeps += 1;
-        cs.pieces += L.n;
-        if (L.phase != kFlatEmit) cs.cand_steps += (unsigned long long)L.n * 3;
-    }
-    if (L.phase == kFlatFirst) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) t.add(L.g2[q], L.st[q].qlo, L.st[q].qhi, L.st[q].cnt);
-        if (L.nt <= out.n_s) {
-            L.gamma = 0.f;
-            L.count = L.nt;
-            flat_start_emit(L);
-        } else {
-            if (CENSUS) cs.searched += 1;
-            L.lo = 0.f;
-            L.hi = 2.f;
-            L.cnt_hi = 1;  // the distance never reaches 2: one supersegment
-            L.it = 0;
-            flat_advance<CENSUS>(L, t, iters, out.n_s, cs);
-        }
-    } else if (L.phase == kFlatSearch) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) t.add(L.g2[q], L.st[q].qlo, L.st[q].qhi, L.st[q].cnt);
-        const int c = L.st[0].cnt;
-        const float mid = 0.5f * (L.lo + L.hi);
-        ++L.it;
-        if (c <= out.n_s) {
-            L.hi = mid;
-            L.cnt_hi = c;
-            if (c == out.n_s) {
-                L.it = iters;  // done
-            }
-        } else {
-            L.lo = mid;
-        }
-        flat_advance<CENSUS>(L, t, iters, out.n_s, cs);
-    } else {
-        // the emission: the open supersegment, the zero tail, count and gamma
-        CompCountQ& s = L.st[0];
-        if (s.open && L.written < out.n_s) {
-            flat_store(out, L.p, L.written, s.fS, L.bt, s.P, s.A, s.L2);
-            ++L.written;
-        }
-        finish_pixel(out, L.p, L.written, L.gamma);
-        if (L.written != L.count) atomicCAS(status, 0u, (unsigned)VDI_ERR_CUDA);
-        L.phase = kFlatIdle;
-    }
+__device__ __forceinline__ bool flat_open(const FlatPair& s) {
+    float nA, u;
+    unpk(s.nA, nA, u);
+    return nA != 0.f;
 }
 
 // Where the flat loop finds its pixels: the list's entries (one request) ...
@@ -2136,7 +2222,9 @@ struct FlatSrcOne {
         if (en.p & 0x80000000u) return false;  // the direct sweep's
         L.p = en.p;
         L.base = en.base;
-        L.n = en.n;
+        L.n = (int)pieces_of(en.n_nt);
+        L.nt = (int)opaque_of(en.n_nt);
+        L.ncol = (int)columns_of(en.n_nt);
         L.f0 = en.f0;
         L.out = out;
         return true;
@@ -2148,115 +2236,183 @@ struct FlatSrcOne {
     }
 };
 
+// Shared memory of a flat CTA: the lanes' bisections, and their next pieces, two groups of four each, copied
+// asynchronously while the groups before them are worked on: a lane's pieces come from L2 or DRAM once per march,
+// and loads into registers left it waiting (25% of the issue slots used, against 8.7 stalls on a load per
+// instruction).  Element i of lane l at i * 128 + l: 16-byte accesses without bank conflicts.
+constexpr int kFlatThreads = 128;
+struct FlatShared {
+    float4 A[2 * 4][kFlatThreads];
+    float4 B[2 * 2][kFlatThreads];  // (b, log2(1 - a)) of two pieces
+    GammaSearch search[kFlatThreads];
+};
+
+// starts the copy of group q of the lane's run (an empty group at its end keeps the count of groups in flight)
+__device__ __forceinline__ void flat_fetch(FlatShared& S, const PiecePool& pool, const FlatLane& L, int q) {
+    if (q * 4 < L.n) {
+        const size_t at = (size_t)L.base + (size_t)q * 4 * L.ncol;
+        const float4* a = pool.A + at;
+        const float4* b = reinterpret_cast<const float4*>(pool.B + at);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) cp_async16(&S.A[(q & 1) * 4 + i][threadIdx.x], a + i);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) cp_async16(&S.B[(q & 1) * 2 + i][threadIdx.x], b + i);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
 // The search and emission of the listed pixels, a lane each (list: [count, next-entry counter, ...]
 // then the entries SRC reads).
 template <bool CENSUS, class SRC>
 __device__ __forceinline__ void flat_loop(const SRC& src, const PiecePool& pool, uint32_t* list, int iters,
-                                          unsigned int* status, CompCensus& cs) {
+                                          unsigned int* status, FlatShared& S, CompCensus& cs) {
+    GammaSearch& sh = S.search[threadIdx.x];
     const uint32_t n_list = list[0];
     const int lane = threadIdx.x & 31;
     FlatLane L;
-    L.phase = kFlatIdle;
     L.out = nullptr;
-    CountTable t;
-    t.n = 0;
-    bool exhausted = false;
-    float4 cA = make_float4(0.f, 0.f, 0.f, 0.f);
-    float2 cB = make_float2(0.f, 0.f);
+    L.p = L.base = 0;
+    L.n = L.nt = L.ncol = 0;
+    L.f0 = 0.f;
+    FlatPair st[kCand / 2];
+    f32x2 g2[kCand / 2];
+    int j = 0, written = 0;
+    float f = 0.f, bt = 0.f;
+    bool has = false, emitting = false, exhausted = false, last = false;
+#pragma unroll
+    for (int w = 0; w < kCand / 2; ++w) {
+        fp_reset(st[w], 0.f);
+        g2[w] = 0ull;
+    }
     while (true) {
-        // idle lanes take the next entries, one atomic per warp (in a list sorted by piece count, the
-        // entries one fetch hands to a warp's lanes have nearly equal counts)
-        const unsigned need = __ballot_sync(0xffffffffu, L.phase == kFlatIdle && !exhausted);
-        if (need) {
-            const int leader = __ffs(need) - 1;
-            uint32_t first = 0;
-            if (lane == leader) first = atomicAdd(list + 1, (uint32_t)__popc(need));
-            first = __shfl_sync(0xffffffffu, first, leader);
-            if ((need >> lane) & 1u) {
-                const uint32_t idx = first + (uint32_t)__popc(need & ((1u << lane) - 1u));
-                if (idx >= n_list) {
-                    exhausted = true;
-                } else if (src.get(idx, L)) {  // (a marked entry leaves the lane idle: it takes another)
-                    L.phase = kFlatFirst;
-                    t.n = 0;
-                    flat_start_count(L, 0.f, 2.f);
-                    if (CENSUS) {
-                        cs.pixels += 1;
-                        cs.records += src.records(L.p);
+        const unsigned act = __ballot_sync(0xffffffffu, has || !exhausted);
+        if (!act) break;
+        // a lane at the end of its march, or without a pixel, waits until VDI_FLAT_END_BATCH lanes (or all
+        // active ones) are there: the divergent end of a march (the replay of bisection levels, the next
+        // march's candidates, a new pixel) runs once for all of them instead of once per lane while the others idle
+        const bool at_end = has ? j >= L.n : !exhausted;
+        const unsigned pend = __ballot_sync(0xffffffffu, at_end);
+        if (pend != 0u && (pend == act || __popc(pend) >= VDI_FLAT_END_BATCH)) {
+            bool count = false, emit = false;  // the next march
+            if (has && at_end) {
+                if (CENSUS) {
+                    cs.sweeps += 1;
+                    cs.pieces += L.n;
+                    if (!emitting) cs.cand_steps += (unsigned long long)L.n * kCand;
+                }
+                if (emitting) {
+                    // the open supersegment, the zero tail, count and gamma
+                    if (flat_open(st[0]) && written < L.out->n_s) {
+                        flat_record(L, st[0], written, bt);
+                        ++written;
+                    }
+                    finish_pixel(*L.out, L.p, written, sh.ghi);
+                    if (written != sh.cnt_hi) atomicCAS(status, 0u, (unsigned)VDI_ERR_CUDA);
+                    has = false;
+                } else {
+                    float k0, k1, k2, k3;
+                    unpk(st[0].kept, k0, k1);
+                    unpk(st[1].kept, k2, k3);
+                    search_end_march(sh, L.nt - (int)k0, L.nt - (int)k1, L.nt - (int)k2, L.nt - (int)k3, L.out->n_s,
+                                     iters, L.nt);
+                    emit = sh.phase == kBisDone;
+                    count = !emit;
+                }
+            }
+            // lanes without a pixel take the next entries, one atomic per warp (in a list sorted by piece
+            // count, the entries one fetch hands to a warp's lanes have nearly equal counts)
+            const unsigned need = __ballot_sync(0xffffffffu, !has && !exhausted);
+            if (need) {
+                const int leader = __ffs(need) - 1;
+                uint32_t first = 0;
+                if (lane == leader) first = atomicAdd(list + 1, (uint32_t)__popc(need));
+                first = __shfl_sync(0xffffffffu, first, leader);
+                if ((need >> lane) & 1u) {
+                    const uint32_t idx = first + (uint32_t)__popc(need & ((1u << lane) - 1u));
+                    if (idx >= n_list) {
+                        exhausted = true;
+                    } else if (src.get(idx, L)) {  // (a marked entry leaves the lane idle: it takes another)
+                        has = true;
+                        if (CENSUS) {
+                            cs.pixels += 1;
+                            cs.records += src.records(L.p);
+                        }
+                        if (L.nt <= L.out->n_s) {  // gamma = 0 meets the budget
+                            sh.ghi = 0.f;
+                            sh.cnt_hi = L.nt;
+                            emit = true;
+                        } else {
+                            if (CENSUS) cs.searched += 1;
+                            // (the distance never reaches 2: one supersegment there)
+                            search_start(sh, L.out->n_s, iters, L.nt, 1, false);
+                            count = true;
+                        }
                     }
                 }
             }
-        }
-        const bool active = L.phase != kFlatIdle;
-        const unsigned act = __ballot_sync(0xffffffffu, active);
-        if (!act) {
-            if (__all_sync(0xffffffffu, exhausted)) break;
-            continue;  // lanes that drew a marked entry draw again
-        }
-        // a lane at the end of its march waits until VDI_FLAT_END_BATCH lanes (or all active ones) are
-        // there: the end of a march (table updates, the replay of bisection levels, the next march's
-        // candidates) runs once for all of them instead of once per lane while the others idle
-        const bool at_end = active && L.j == L.n;
-        const unsigned pend = __ballot_sync(0xffffffffu, at_end);
-        if (pend != 0u && (pend == act || __popc(pend) >= VDI_FLAT_END_BATCH)) {
-            if (at_end) flat_end_march<CENSUS>(L, t, *L.out, iters, status, cs);
+            if (count || emit) {
+                emitting = emit;
+                const float ge = __fmul_rn(sh.ghi, sh.ghi);
+#pragma unroll
+                for (int w = 0; w < kCand / 2; ++w) {
+                    g2[w] = emit ? pk(ge) : pk(sh.g2[2 * w], sh.g2[2 * w + 1]);
+                    fp_reset(st[w], L.f0);
+                }
+                j = 0;
+                f = L.f0;
+                written = 0;
+                bt = 0.f;
+                last = emit && L.out->n_s <= 1;
+                flat_fetch(S, pool, L, 0);
+                flat_fetch(S, pool, L, 1);
+            }
             continue;
         }
-        if (!active || at_end) continue;
-        // one piece of the lane's march
-        if (L.j == 0) {
-            cA = pool.A[L.base];
-            cB = pool.B[L.base];
-        }
-        Piece x;
-        x.f = L.f;
-        x.b = cB.x;
-        x.P[0] = cA.x;
-        x.P[1] = cA.y;
-        x.P[2] = cA.z;
-        x.a = cA.w;
-        x.lgT = cB.y;
-        if (L.j + 1 < L.n) {
-            cA = pool.A[L.base + L.j + 1];
-            cB = pool.B[L.base + L.j + 1];
-        }
-        // one instruction stream for counting and emitting lanes: candidate 0 carries the budget (none
-        // while counting) and, emitting, writes the supersegment a termination closes -- EmitVisitor's
-        // decisions, in select form; candidates 1 and 2 only count
-        {
-            const bool emitting = L.phase == kFlatEmit;
-            const int cap = emitting ? L.out->n_s : INT_MAX;
-            CompCountQ& s = L.st[0];
-            float q = 0.f;
-            const bool crit = s.open && s.cnt < cap &&
-                              criterion_q(s.P, s.A, s.L2, piece_ratio(s, x), x.P, L.g2[0], q);
-            if (emitting && crit && L.written < cap) {
-                flat_store(*L.out, L.p, L.written, s.fS, L.bt, s.P, s.A, s.L2);
-                ++L.written;
+        if (!has || at_end) continue;
+        // four pieces of the lane's march
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        const int q = j >> 2, stop = min(L.n, j + 4);
+#pragma unroll 1
+        for (; j < stop; ++j) {
+            const float4 A = S.A[j & 7][threadIdx.x];
+            const float2 B = reinterpret_cast<const float2*>(&S.B[(j >> 1) & 3][threadIdx.x])[j & 1];
+            const float b = B.x;
+            const bool opaque = A.w > 0.f;
+            const PieceX x{{pk(A.x), pk(A.y), pk(A.z)},
+                           pk(-A.w),
+                           pk(fmaxf(B.y, -1e34f)),
+                           pk(f),
+                           pk(__fsub_rn(b, f)),
+                           pk(opaque ? 1.f : 0.f)};
+            // one instruction stream for counting and emitting lanes: an emitting lane's first candidate carries
+            // the budget and writes the supersegment a termination closes
+            const f32x2 k = fp_keep(st[0], x, g2[0], last);
+            if (emitting) {
+                float k0, u1;
+                unpk(k, k0, u1);
+                if (k0 == 0.f && flat_open(st[0])) {
+                    if (written < L.out->n_s) flat_record(L, st[0], written, bt);
+                    ++written;
+                    last = written + 1 >= L.out->n_s;
+                }
+                bt = opaque ? b : bt;
             }
-            s.qhi = crit ? fminf(s.qhi, q) : s.qhi;
-            s.qlo = (s.open && !crit) ? fmaxf(s.qlo, q) : s.qlo;
-            const bool opaque = x.a > 0.f;
-            const bool fresh = opaque && (!s.open || crit);
-            const bool absorbing = s.open && !crit;
-            L.bt = (fresh || (absorbing && opaque)) ? x.b : L.bt;
-            apply_step(s, x, StepSel{fresh, crit && !opaque});
-            L.nt += opaque;
-            cq_step_select(L.st[1], x, L.g2[1]);
-            cq_step_select(L.st[2], x, L.g2[2]);
+            fp_apply(st[0], x, k);
+#pragma unroll
+            for (int w = 1; w < kCand / 2; ++w) fp_apply(st[w], x, fp_keep(st[w], x, g2[w], false));
+            f = b;
         }
-        L.f = x.b;
-        ++L.j;
+        flat_fetch(S, pool, L, q + 2);
     }
 }
 
 template <bool CENSUS>
-__global__ void __launch_bounds__(128) composite_flat_kernel(const __grid_constant__ CompArgs a,
-                                                             const __grid_constant__ PiecePool pool,
-                                                             uint32_t* list) {
+__global__ void __launch_bounds__(kFlatThreads, VDI_FLAT_MIN_BLOCKS) composite_flat_kernel(
+    const __grid_constant__ CompArgs a, const __grid_constant__ PiecePool pool, uint32_t* list) {
+    __shared__ FlatShared S;
     CompCensus cs;
     const FlatSrcOne src{reinterpret_cast<const FlatEntry*>(list + 4), &a.out, a.pe, a.k};
-    flat_loop<CENSUS>(src, pool, list, a.iters, a.status, cs);
+    flat_loop<CENSUS>(src, pool, list, a.iters, a.status, S, cs);
     if (CENSUS) census_flush(cs, reinterpret_cast<WsHeader*>(a.status)->counters);
 }
 
@@ -2286,7 +2442,7 @@ __global__ void __launch_bounds__(256) list_hist_kernel(const uint32_t* __restri
     const E* en = reinterpret_cast<const E*>(list + HW);
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const E e = en[i];
-        if (!(e.p & 0x80000000u)) atomicAdd(&h[sort_bin(e.n)], 1u);
+        if (!(e.p & 0x80000000u)) atomicAdd(&h[sort_bin(pieces_of(e.n_nt))], 1u);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < kSortBins; i += blockDim.x)
@@ -2342,7 +2498,7 @@ __global__ void __launch_bounds__(256) list_scatter_kernel(const uint32_t* __res
         }
         const unsigned act = __ballot_sync(0xffffffffu, take);
         if (take) {
-            const uint32_t b = sort_bin(e.n);
+            const uint32_t b = sort_bin(pieces_of(e.n_nt));
             const unsigned grp = __match_any_sync(act, b);
             const int leader = __ffs(grp) - 1;
             uint32_t slot = 0;
@@ -2412,7 +2568,7 @@ __device__ __forceinline__ int request_of(const BatchArgs& a, uint32_t item) {
 // pixels, a lane each, each into its request's output; composite_batched_
 // marked_kernel sweeps the pixels listed for the direct path.
 struct BatchEntry {
-    uint32_t p, base, n;
+    uint32_t p, base, n_nt;  // as FlatEntry's
     float f0;
     uint32_t req, pad0, pad1, pad2;
 };
@@ -2435,52 +2591,29 @@ __device__ __forceinline__ void batch_push(uint32_t* list, bool flag, const Batc
     if (flag) reinterpret_cast<BatchEntry*>(list + 8)[base + __popc(m & ((1u << lane) - 1u))] = en;
 }
 
-template <int PREC>
-__global__ void __launch_bounds__(kStageWarps * 32, 1) composite_batched_build_kernel(
+template <int NW, int PREC>
+__global__ void __launch_bounds__(kStageWarps * 32) composite_batched_build_kernel(
     const __grid_constant__ BatchArgs a, const __grid_constant__ BatchBuildArgs bb) {
-    extern __shared__ __align__(16) unsigned char stage_smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    StageSmem& S = reinterpret_cast<StageSmem*>(stage_smem)[warp];
+    constexpr int RMAX = NW == 1 ? kStageRSmall : kStageRMax, RMIN = NW == 1 ? 0 : kStageRSmall;
+    __shared__ BuildShared<NW, RMAX> sh;
     while (true) {
-        uint32_t item = 0;
-        if (lane == 0) item = bb.item0 + atomicAdd(bb.counter, 1u);
-        item = __shfl_sync(0xffffffffu, item, 0);
+        const uint32_t item = bb.item0 + next_item<NW>(bb.counter + (NW == 1 ? 0 : 1), &sh.item);
         if (item >= bb.item1) break;
         const int rq = request_of(a, item);
         const ReqDev& r = a.reqs[rq];
         const uint32_t base = (item - r.item_begin) * 32u;
-        BatchEntry mine{0u, 0u, 0u, 0.f, (uint32_t)rq, 0u, 0u, 0u};
-        bool have = false;
+        BatchPixel px;
         if (r.schedule == VDI_SCHED_STAGED) {
-            for (int col = 0; col < 32; ++col) {
-                const uint32_t p = base + (uint32_t)col;
-                if (p >= r.npix) break;
-                PoolRun run{bb.list + 2, bb.pool.cap, 0u};
-                int n = 0, nt = 0;
-                float f0 = 0.f;
-                const bool ok = stage_pixel<PREC, true>(a.pes + r.pe_begin, r.k, p, S, bb.pool.A, bb.pool.B,
-                                                        0x7FFFFFFF, n, nt, f0, &run);
-                if (lane == col) {
-                    if (!ok || n < 0) {
-                        mine.p = p | 0x80000000u;
-                        have = true;
-                    } else if (n == 0) {
-                        finish_pixel(r.out, p, 0, 0.f);  // no record: an empty list
-                    } else {
-                        mine.p = p;
-                        mine.base = run.base;
-                        mine.n = (uint32_t)n;
-                        mine.f0 = f0;
-                        have = true;
-                    }
-                }
-            }
+            if (!build_batch<NW, PREC, RMIN, RMAX>(a.pes + r.pe_begin, r.k, base, r.npix, r.out, bb.pool, pool_used(bb.list),
+                                                   sh.stage[NW == 1 ? threadIdx.x >> 5 : 0], sh.tot, &sh.base, px))
+                continue;
+            if (NW > 1 && threadIdx.x >= 32) continue;
         } else {
-            const uint32_t p = base + (uint32_t)lane;
-            have = p < r.npix;
-            mine.p = p | 0x80000000u;
+            if (NW > 1) continue;
+            const uint32_t p = base + (threadIdx.x & 31);
+            px = BatchPixel{p < r.npix, p | 0x80000000u, 0u, 0u, 0.f};
         }
-        batch_push(bb.list, have, mine);
+        batch_push(bb.list, px.have, BatchEntry{px.p, px.base, px.n_nt, px.f0, (uint32_t)rq, 0u, 0u, 0u});
     }
 }
 
@@ -2492,7 +2625,9 @@ struct FlatSrcBatch {
         if (en.p & 0x80000000u) return false;  // the direct sweep's
         L.p = en.p;
         L.base = en.base;
-        L.n = en.n;
+        L.n = (int)pieces_of(en.n_nt);
+        L.nt = (int)opaque_of(en.n_nt);
+        L.ncol = (int)columns_of(en.n_nt);
         L.f0 = en.f0;
         L.out = &reqs[en.req].out;
         return true;
@@ -2500,12 +2635,12 @@ struct FlatSrcBatch {
     __device__ __forceinline__ unsigned long long records(uint32_t) const { return 0; }
 };
 
-__global__ void __launch_bounds__(128) composite_batched_flat_kernel(const __grid_constant__ BatchArgs a,
-                                                                     const __grid_constant__ PiecePool pool,
-                                                                     uint32_t* list) {
+__global__ void __launch_bounds__(kFlatThreads, VDI_FLAT_MIN_BLOCKS) composite_batched_flat_kernel(
+    const __grid_constant__ BatchArgs a, const __grid_constant__ PiecePool pool, uint32_t* list) {
+    __shared__ FlatShared S;
     CompCensus cs;
     const FlatSrcBatch src{reinterpret_cast<const BatchEntry*>(list + 8), a.reqs};
-    flat_loop<false>(src, pool, list, a.iters, a.status, cs);
+    flat_loop<false>(src, pool, list, a.iters, a.status, S, cs);
 }
 
 template <int P, int PREC>
@@ -2555,13 +2690,25 @@ static int device_sms() {
     return sms;
 }
 
-// Workspace of the staged path: [header][batch counter][overflow count, pad,
-// entries][piece buffers], for `batches` 32-pixel batches and `entries`
-// overflow entries of `entry_bytes`.
-static size_t stage_ctas(uint64_t batches) {
-    const uint64_t need = (batches + kStageWarps - 1) / kStageWarps;
-    const uint64_t sms = (uint64_t)device_sms();
-    return (size_t)(need < sms ? (need > 0 ? need : 1) : sms);
+// CTAs of a build launch over `batches` 32-pixel batches
+template <int NW, typename K>
+static cudaError_t build_ctas(K kernel, uint64_t batches, unsigned& ctas) {
+    int per_sm = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kStageWarps * 32, 0);
+    const uint64_t need = NW == 1 ? (batches + kStageWarps - 1) / kStageWarps : batches;
+    const uint64_t most = (uint64_t)device_sms() * (uint64_t)(per_sm > 0 ? per_sm : 1);
+    ctas = (unsigned)(need < most ? (need > 0 ? need : 1) : most);
+    return e;
+}
+
+template <int NW, int PREC>
+static cudaError_t launch_build(bool census, const CompArgs& a, const BuildArgs& ba, cudaStream_t st) {
+    auto kb = census ? composite_build_kernel<NW, PREC, true> : composite_build_kernel<NW, PREC, false>;
+    unsigned ctas = 0;
+    cudaError_t e = build_ctas<NW>(kb, (ba.p1 - ba.p0 + 31) / 32, ctas);
+    if (e != cudaSuccess) return e;
+    kb<<<ctas, kStageWarps * 32, 0, st>>>(a, ba);
+    return cudaGetLastError();
 }
 
 // pixels per chunk of the pooled staged path that the queried workspace holds at the stage's worst case
@@ -2662,10 +2809,7 @@ static cudaError_t launch_staged_pool(bool census, const CompArgs& a, void* work
     ba.pool.cap = (uint32_t)cap;
     ba.pool.A = reinterpret_cast<float4*>(base + head + list_bytes);
     ba.pool.B = reinterpret_cast<float2*>(base + head + list_bytes + cap * sizeof(float4));
-    const size_t sm = kStageWarps * sizeof(StageSmem);
-    auto kb = census ? composite_build_kernel<PREC, true> : composite_build_kernel<PREC, false>;
-    cudaError_t e = cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     const int P = tree_leaves(a.k);
     for (uint64_t p0 = 0; p0 < npix; p0 += chunk) {
         const uint64_t p1 = p0 + chunk < npix ? p0 + chunk : npix;
@@ -2674,8 +2818,8 @@ static cudaError_t launch_staged_pool(bool census, const CompArgs& a, void* work
         e = cudaMemsetAsync(ba.counter, 0, 256, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(ba.list, 0, 16, st);
         if (e != cudaSuccess) return e;
-        kb<<<(unsigned)stage_ctas((p1 - p0 + 31) / 32), kStageWarps * 32, sm, st>>>(a, ba);
-        e = cudaGetLastError();
+        e = launch_build<1, PREC>(census, a, ba, st);
+        if (e == cudaSuccess) e = launch_build<kStageWarps, PREC>(census, a, ba, st);
         if (e == cudaSuccess) e = launch_flat<PREC>(census, a, ba.pool, ba.list, p1 - p0, st, VDI_FLAT_CTAS_PER_SM);
         if (e == cudaSuccess) {
             if (P == 16) e = launch_marked<0, 16, PREC>(census, a, ba.list, p1 - p0, st);
@@ -2872,10 +3016,7 @@ static cudaError_t launch_batched(const BatchArgs& a, const BatchHeader* hd, con
     bb.pool.cap = (uint32_t)cap;
     bb.pool.A = reinterpret_cast<float4*>(base + fixed);
     bb.pool.B = reinterpret_cast<float2*>(base + fixed + cap * sizeof(float4));
-    const size_t sm = kStageWarps * sizeof(StageSmem);
-    cudaError_t e = cudaFuncSetAttribute(composite_batched_build_kernel<PREC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     const int P = tree_leaves((int)hd->max_k);
     const size_t smd = P == 16 ? heads_smem_bytes<16>(128) : (P == 32 ? heads_smem_bytes<32>(128)
                                                                         : heads_smem_bytes<64>(128));
@@ -2908,7 +3049,13 @@ static cudaError_t launch_batched(const BatchArgs& a, const BatchHeader* hd, con
         e = cudaMemsetAsync(bb.counter, 0, 256, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(bb.list, 0, 32, st);
         if (e != cudaSuccess) return e;
-        composite_batched_build_kernel<PREC><<<(unsigned)stage_ctas(item - item0), kStageWarps * 32, sm, st>>>(a, c);
+        unsigned ctas = 0;
+        e = build_ctas<1>(composite_batched_build_kernel<1, PREC>, item - item0, ctas);
+        if (e != cudaSuccess) return e;
+        composite_batched_build_kernel<1, PREC><<<ctas, kStageWarps * 32, 0, st>>>(a, c);
+        e = build_ctas<kStageWarps>(composite_batched_build_kernel<kStageWarps, PREC>, item - item0, ctas);
+        if (e != cudaSuccess) return e;
+        composite_batched_build_kernel<kStageWarps, PREC><<<ctas, kStageWarps * 32, 0, st>>>(a, c);
         uint64_t b = (uint64_t)device_sms() * (uint64_t)(per_sm > 0 ? per_sm : 1);
         const uint64_t need = (pixels + 127) / 128;
         if (b > need) b = need > 0 ? need : 1;
