@@ -147,29 +147,52 @@ struct U128 {
 };
 
 __device__ __forceinline__ void u128_add(U128& s, const U128& x) {
-    const unsigned long long lo = s.lo + x.lo;
-    s.hi += x.hi + (lo < s.lo ? 1ull : 0ull);
-    s.lo = lo;
+    asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(s.lo), "+l"(s.hi) : "l"(x.lo), "l"(x.hi));
 }
 
 __device__ __forceinline__ void u128_sub(U128& s, const U128& x) {
-    const unsigned long long lo = s.lo - x.lo;
-    s.hi -= x.hi + (s.lo < x.lo ? 1ull : 0ull);
-    s.lo = lo;
+    asm("sub.cc.u64 %0, %0, %2;\n\tsubc.u64 %1, %1, %3;" : "+l"(s.lo), "+l"(s.hi) : "l"(x.lo), "l"(x.hi));
 }
 
-// v in [0, 2^56] as fixed point: exact for v >= 2^-41 (the 24-bit significand
-// fits in the 64 fraction bits), truncated below
+// s + x, or s - x where neg is all ones (s + ~x + 1), without a branch
+__device__ __forceinline__ void u128_add_signed(U128& s, const U128& x, unsigned long long neg) {
+    asm("{\n\t.reg .u64 t;\n\tadd.cc.u64 t, %4, %4;\n\taddc.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;\n\t}"
+        : "+l"(s.lo), "+l"(s.hi)
+        : "l"(x.lo ^ neg), "l"(x.hi ^ neg), "l"(neg));
+}
+
+// The conversions between FP32 and this format in 32-bit integer operations: the hardware's conversions to and from
+// 64-bit integers run on the FP64 pipe, 2 lanes an SM on this chip (16 cycles a warp for each, 8 of them per bound
+// and per piece: more than half of the pooled build's time).
+
+// v in [0, 2^56] as fixed point: the significand shifted to its place, exact for v >= 2^-41 (its 24 bits fit the
+// 64 fraction bits), truncated below
 __device__ __forceinline__ U128 to_fixed(float v) {
-    const float ip = truncf(v);
+    const uint32_t bits = __float_as_uint(v);
+    const int sh = (int)(bits >> 23) - 86;  // of the significand's last bit, from the last fraction bit
+    const uint32_t m = (bits & 0x7FFFFFu) | 0x800000u;
+    const uint32_t lo = sh < 0 ? (sh > -32 ? m >> -sh : 0u) : m << (sh & 31);
+    const uint32_t hi = sh < 0 ? 0u : __funnelshift_l(m, 0u, sh & 31);
+    const int w = sh < 0 ? 0 : sh >> 5;  // the 32-bit word that lo falls in (at most 3)
+    const uint32_t w0 = w == 0 ? lo : 0u, w1 = w == 0 ? hi : (w == 1 ? lo : 0u);
+    const uint32_t w2 = w == 1 ? hi : (w == 2 ? lo : 0u), w3 = w == 2 ? hi : (w == 3 ? lo : 0u);
     U128 r;
-    r.hi = __float2ull_rz(ip);
-    r.lo = __float2ull_rz(__fmul_rn(__fsub_rn(v, ip), 18446744073709551616.f));
+    r.lo = (unsigned long long)w1 << 32 | w0;
+    r.hi = (unsigned long long)w3 << 32 | w2;
     return r;
 }
 
+// x rounded to nearest even: its top 32 bits, the rest folded into the last of them, converted and scaled
+__device__ __forceinline__ float u64_to_float(unsigned long long x) {
+    const uint32_t hi = (uint32_t)(x >> 32), lo = (uint32_t)x;
+    const int z = __clz(hi);  // 32 where hi is 0
+    const uint32_t top = hi ? __funnelshift_l(lo, hi, z) : lo;
+    const uint32_t sticky = hi && (lo << (z & 31)) != 0u ? 1u : 0u;
+    return __fmul_rn(__uint2float_rn(top | sticky), __uint_as_float((uint32_t)(159 - z) << 23));  // 2^(32 - z)
+}
+
 __device__ __forceinline__ float from_fixed(const U128& s) {
-    return __fmaf_rn(__ull2float_rn(s.lo), 5.421010862427522e-20f, __ull2float_rn(s.hi));
+    return __fmaf_rn(u64_to_float(s.lo), 5.421010862427522e-20f, u64_to_float(s.hi));
 }
 
 // Clamp of a record's extinction terms (per unit depth): a record shorter than
@@ -207,6 +230,42 @@ __device__ __forceinline__ Contrib contrib(const RecC& x, float f, float b) {
         r.M = to_fixed(mu);
 #pragma unroll
         for (int q = 0; q < 3; ++q) r.MC[q] = to_fixed(fminf(fmaxf(__fmul_rn(mu, __fmul_rn(col[q], ia)), 0.f), kMuMax));
+    }
+    return r;
+}
+
+// A record's terms before their conversion to fixed point, as contrib computes them: extinction mu and mu times the
+// colour (all 0 for a transparent record), or -1 and the colour of an opaque one.
+__device__ __forceinline__ float4 record_terms(const RecC& x, float f, float b) {
+    const float col[3] = {x.c.x, x.c.y, x.c.z};
+    float t[3] = {0.f, 0.f, 0.f}, mu = 0.f;
+    if (rec_opaque(x)) {
+        mu = -1.f;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) t[q] = fminf(fmaxf(col[q], 0.f), kMuMax);
+    } else if (x.c.w > 0.f) {
+        const float ia = rcp_approx(x.c.w);
+        mu = fminf(__fmul_rn(x.tau, rcp_approx(__fsub_rn(b, f))), kMuMax);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) t[q] = fminf(fmaxf(__fmul_rn(mu, __fmul_rn(col[q], ia)), 0.f), kMuMax);
+    }
+    return make_float4(t[0], t[1], t[2], mu);
+}
+
+template <bool OPQ>
+__device__ __forceinline__ Contrib contrib_of(const float4& t) {
+    Contrib r;
+    const bool op = OPQ && t.w < 0.f;
+    r.op = op ? 1 : 0;
+    const float v[3] = {t.x, t.y, t.z};
+    r.M = to_fixed(op ? 0.f : t.w);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const U128 x = to_fixed(v[q]);
+        u128_zero(r.MC[q]);
+        u128_zero(r.OC[q]);
+        if (op) r.OC[q] = x;
+        else r.MC[q] = x;
     }
     return r;
 }
@@ -1043,10 +1102,14 @@ __device__ __forceinline__ void finish_pixel(const OutDev& out, uint32_t p, int 
 // A pixel is built by one warp when its 32-pixel batch's lists are short, by a CTA of four when they are long:
 // the steps are chains of dependent shared-memory reads, so what counts is the warps an SM holds.  A warp's
 // stage of 1024 records (20 KB, a 172 KB CTA of 8 warps) left 8 warps per SM, 17% of the issue slots used; four
-// warps on such a stage make 40, and short lists take a stage of 320 records (7 KB) each.
+// warps on such a stage make 40, and short lists take a stage of 288 records (11 KB) each.
 constexpr int kStageRMax = 1024;   // records per pixel held by the largest stage
-constexpr int kStageRSmall = 320;  // records per pixel of a batch that single warps build
+constexpr int kStageRSmall = 288;  // records per pixel of a batch that single warps build
 constexpr int kStageWarps = 4;     // warps per CTA, of either kind
+
+#ifndef VDI_BUILD_MIN_BLOCKS
+#define VDI_BUILD_MIN_BLOCKS 5
+#endif
 
 struct ScanState;
 
@@ -1054,6 +1117,7 @@ template <int RMAX>
 struct StageSmem {
     uint16_t pay[2][2 * RMAX];      // bounds: (valid record << 1) | is_back
     float2 rfb[RMAX];               // bounds of the valid records
+    float4 term[RMAX];              // their terms (record_terms)
     uint32_t rloc[RMAX];            // (PE << 16) | index in the PE's list, of the valid records
     uint32_t pref[VDI_MAX_PE + 1];  // records before PE e
     uint32_t vpref[VDI_MAX_PE + 1]; // valid records before PE e
@@ -1078,8 +1142,7 @@ __device__ __forceinline__ bool group_any(bool v) {
 
 template <int RMAX>
 __device__ __forceinline__ float bound_key(const StageSmem<RMAX>& S, uint32_t w) {
-    const float2 fb = S.rfb[w >> 1];
-    return (w & 1u) ? fb.y : fb.x;
+    return reinterpret_cast<const float*>(S.rfb)[w];  // w = 2 record + is_back
 }
 
 __device__ __forceinline__ uint32_t warp_incl_scan_u32(uint32_t v) {
@@ -1144,17 +1207,42 @@ __device__ __forceinline__ ScanState shfl_up_state(const ScanState& v, int d) {
     return r;
 }
 
-// applies bound w (sorted position i) to the state
-template <int PREC, bool OPQ, int RMAX>
-__device__ __forceinline__ void stage_apply(const PeIn* pe, const StageSmem<RMAX>& S, uint32_t w, ScanState& a) {
-    const uint32_t c = w >> 1;
-    const uint32_t loc = S.rloc[c];
-    const int e = (int)(loc >> 16);
-    const float2 fb = S.rfb[c];
-    const Contrib x = contrib(load_rec<PREC>(pe[e], S.off[e] + (loc & 0xFFFFu)), fb.x, fb.y);
-    if (w & 1u) sums_update<false, OPQ>(a.s, x);
-    else sums_update<true, OPQ>(a.s, x);
-    a.xr ^= c;
+// applies bound w, of the record with terms t, to the state
+template <bool OPQ>
+__device__ __forceinline__ void stage_apply(uint32_t w, const float4& t, ScanState& a) {
+    const Contrib x = contrib_of<OPQ>(t);
+    const int sign = 1 - 2 * (int)(w & 1u);
+    const unsigned long long neg = (unsigned long long)((long long)sign >> 1);  // fronts add, backs subtract
+    u128_add_signed(a.s.M, x.M, neg);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        u128_add_signed(a.s.MC[q], x.MC[q], neg);
+        if (OPQ) u128_add_signed(a.s.OC[q], x.OC[q], neg);
+    }
+    if (OPQ) a.s.nop += sign * x.op;
+    a.s.nact += sign;
+    a.xr ^= w >> 1;
+}
+
+// Walks the sorted bounds [i0, i1) of the stage: visit(w, terms, key, next key, there is a next), each bound's values
+// read a bound ahead of their use and its place in the order two ahead (the three reads depend on each other).
+template <int RMAX, typename F>
+__device__ __forceinline__ void stage_walk(const StageSmem<RMAX>& S, const uint16_t* srt, uint32_t E, uint32_t i0,
+                                           uint32_t i1, F&& visit) {
+    if (i0 >= i1) return;
+    uint32_t w = srt[i0], w1 = srt[min(i0 + 1, E - 1)];
+    float key = bound_key(S, w);
+    float4 t = S.term[w >> 1];
+    for (uint32_t i = i0; i < i1; ++i) {
+        const uint32_t w2 = srt[min(i + 2, E - 1)];
+        const float key1 = bound_key(S, w1);
+        const float4 t1 = S.term[w1 >> 1];
+        visit(w, t, key, key1, i + 1 < E);
+        w = w1;
+        w1 = w2;
+        key = key1;
+        t = t1;
+    }
 }
 
 // Where phase G writes a pixel's pieces: column `col` of its batch's part of the pool, rows of 4 pieces by
@@ -1179,15 +1267,14 @@ __device__ __forceinline__ void stage_scan(const PeIn* pe, StageSmem<RMAX>& S, S
                                            float& f0) {
     constexpr uint32_t T = 32 * NW;
     const int lane = threadIdx.x & 31, rank = group_rank<NW>();
-    const uint32_t chunk = (E + T - 1) / T;
+    const uint32_t chunk = ((E + T - 1) / T) | 1u;  // (odd: the threads' reads of their chunks spread over the banks)
     const uint32_t i0 = min(E, rank * chunk), i1 = min(E, i0 + chunk);
     ScanState loc;
     scan_reset(loc);
-#pragma unroll 4
-    for (uint32_t i = i0; i < i1; ++i) {
-        stage_apply<PREC, OPQ>(pe, S, srt[i], loc);
-        if (i + 1 < E && bound_key(S, srt[i]) < bound_key(S, srt[i + 1])) ++loc.nb;
-    }
+    stage_walk(S, srt, E, i0, i1, [&](uint32_t w, const float4& t, float key, float next, bool more) {
+        stage_apply<OPQ>(w, t, loc);
+        if (more && key < next) ++loc.nb;
+    });
     // exclusive prefix of the threads' totals
     ScanState inc = loc;
 #pragma unroll
@@ -1220,11 +1307,9 @@ __device__ __forceinline__ void stage_scan(const PeIn* pe, StageSmem<RMAX>& S, S
     // the pieces: after bound i the active set is that of [key_i, key_{i+1}]
     uint32_t my_nt = 0;
     uint32_t row = st.nb;
-    for (uint32_t i = i0; i < i1; ++i) {
-        stage_apply<PREC, OPQ>(pe, S, srt[i], st);
-        if (i + 1 >= E) break;
-        const float t = bound_key(S, srt[i]), t1 = bound_key(S, srt[i + 1]);
-        if (!(t < t1)) continue;
+    stage_walk(S, srt, E, i0, i1, [&](uint32_t w, const float4& term, float t, float t1, bool more) {
+        stage_apply<OPQ>(w, term, st);
+        if (!more || !(t < t1)) return;
         bool whole = false;
         RecC wc{make_float4(0.f, 0.f, 0.f, 0.f), 0.f};
         if (st.s.nact == 1) {
@@ -1244,7 +1329,7 @@ __device__ __forceinline__ void stage_scan(const PeIn* pe, StageSmem<RMAX>& S, S
         out.B[at] = make_float2(x.b, x.lgT);
         my_nt += x.a > 0.f;
         ++row;
-    }
+    });
     my_nt = __reduce_add_sync(0xffffffffu, my_nt);
     npieces = (int)total_pieces;
     f0 = bound_key(S, srt[0]);
@@ -1301,8 +1386,13 @@ __device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem<RMAX>& 
         load_fb<PREC>(pe[lo], S.off[lo] + j, f, b);
         S.rfb[r] = make_float2(f, b);
         S.rloc[r] = ((uint32_t)lo << 16) | j;
-        if (b > f) opaque |= rec_opaque(load_rec<PREC>(pe[lo], S.off[lo] + j));
-        else empty = true;
+        if (b > f) {
+            const RecC x = load_rec<PREC>(pe[lo], S.off[lo] + j);
+            opaque |= rec_opaque(x);
+            S.term[r] = record_terms(x, f, b);
+        } else {
+            empty = true;
+        }
     }
     uint32_t nv = R;
     if (group_any<NW>(empty)) {
@@ -1314,12 +1404,14 @@ __device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem<RMAX>& 
                 const uint32_t r = r0 + lane;
                 const float2 fb = r < R ? S.rfb[r] : make_float2(0.f, 0.f);
                 const uint32_t loc = r < R ? S.rloc[r] : 0u;
+                const float4 term = r < R ? S.term[r] : make_float4(0.f, 0.f, 0.f, 0.f);
                 const bool valid = fb.y > fb.x;
                 const unsigned m = __ballot_sync(0xffffffffu, valid);
                 if (valid) {
                     const uint32_t c = n + __popc(m & ((1u << lane) - 1u));
                     S.rfb[c] = fb;
                     S.rloc[c] = loc;
+                    S.term[c] = term;
                 }
                 n += __popc(m);
                 __syncwarp();
@@ -1365,7 +1457,7 @@ __device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem<RMAX>& 
         uint16_t* outp = S.pay[src ^ 1];
         const int span = 2 << r;
         const int ngroups = (k + span - 1) / span;
-        const uint32_t per = (E + T - 1) / T;
+        const uint32_t per = ((E + T - 1) / T) | 1u;  // (odd, as stage_scan's)
         uint32_t o = min(E, rank * per);
         const uint32_t o_end = min(E, o + per);
         while (o < o_end) {
@@ -2075,7 +2167,7 @@ __device__ __forceinline__ uint32_t next_item(unsigned int* counter, uint32_t* s
 }
 
 template <int NW, int PREC, bool CENSUS>
-__global__ void __launch_bounds__(kStageWarps * 32) composite_build_kernel(const __grid_constant__ CompArgs a,
+__global__ void __launch_bounds__(kStageWarps * 32, VDI_BUILD_MIN_BLOCKS) composite_build_kernel(const __grid_constant__ CompArgs a,
                                                                           const __grid_constant__ BuildArgs ba) {
     constexpr int RMAX = NW == 1 ? kStageRSmall : kStageRMax, RMIN = NW == 1 ? 0 : kStageRSmall;
     __shared__ BuildShared<NW, RMAX> sh;
@@ -2592,7 +2684,7 @@ __device__ __forceinline__ void batch_push(uint32_t* list, bool flag, const Batc
 }
 
 template <int NW, int PREC>
-__global__ void __launch_bounds__(kStageWarps * 32) composite_batched_build_kernel(
+__global__ void __launch_bounds__(kStageWarps * 32, VDI_BUILD_MIN_BLOCKS) composite_batched_build_kernel(
     const __grid_constant__ BatchArgs a, const __grid_constant__ BatchBuildArgs bb) {
     constexpr int RMAX = NW == 1 ? kStageRSmall : kStageRMax, RMIN = NW == 1 ? 0 : kStageRSmall;
     __shared__ BuildShared<NW, RMAX> sh;
