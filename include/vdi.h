@@ -166,7 +166,7 @@ vdi_status vdi_workspace_status(const void* workspace, vdi_stream stream);
  *   pixel's pieces (search marches plus the emitting sweep), [3] pieces
  *   visited over those sweeps, [4] state-machine steps (pieces x gamma
  *   candidates), [5] input records, [6] bisection levels answered by the
- *   decision intervals of earlier marches, [7] unused.
+ *   decision intervals of earlier marches (direct sweeps), [7] unused.
  * The census runs a separately compiled variant of the kernel; without the
  * flag nothing is counted. */
 vdi_status vdi_workspace_counters(const void* workspace, uint64_t counters[8], vdi_stream stream);
@@ -303,9 +303,10 @@ size_t vdi_gen_batch_table_bytes(const vdi_gen_request* reqs, int32_t n);
 vdi_status vdi_gen_batch_table_pack(const vdi_gen_request* reqs, int32_t n, const vdi_params* params,
                                     void* host_table, size_t bytes);
 /* Workspace bytes for a packed table: 512 bytes of status and counter, the
- * prefix sums' partial sums (8 bytes per 4096 pixels per PE) and the sample
- * cache of vdi_generate_workspace (the search re-marches the volume when the
- * workspace has no room for it; same result). */
+ * prefix sums' partial sums (8 bytes per 4096 pixels per PE), the sample
+ * cache of vdi_generate_workspace and each (PE, ray)'s recorded span (8 bytes).
+ * Without room for the cache the search re-marches the volume, without room
+ * for the spans emission marches every sample (same results). */
 size_t vdi_generate_batched_workspace(const void* host_table);
 /* Generates every request's k compact sub-VDIs: one persistent launch in
  * which CTAs take (request, PE, 16 x 4-pixel tile) items from an atomic
@@ -361,14 +362,15 @@ vdi_status vdi_generate_static_scratch(const vdi_brick* bricks, int32_t k, const
  * at most n_s supersegments are written front to back with a zero tail.
  * params->schedule (all give the same result, bit for bit):
  *   0 automatic (VDI_SCHED_LANE for k <= 8, else VDI_SCHED_STAGED);
- *   VDI_SCHED_STAGED (4, the pooled schedule): a warp builds the pieces of
- *     32 pixels, one pixel at a time with all its lanes (coalesced loads of
- *     the K lists, a stable merge of their bounds, an exact prefix scan of
- *     the records' terms), writes each pixel's pieces as one run of a pool in
- *     the workspace and lists the pixel; a second launch runs the search and
- *     the emission of every listed pixel, one lane each, lanes taking new
- *     pixels as they finish; pixels with more than 1024 records or lists out
- *     of depth order are composited by a direct sweep in a third launch.  The
+ *   VDI_SCHED_STAGED (4, the pooled schedule): a warp (a CTA of four where a
+ *     list of the 32 is long) builds the pieces of 32 pixels, one pixel at a
+ *     time with all its lanes (coalesced loads of the K lists, a stable merge
+ *     of their bounds, an exact prefix scan of the records' terms) into the
+ *     batch's part of a pool in the workspace and lists the pixels; another
+ *     launch runs the search and the emission of every listed pixel, one lane
+ *     each, lanes taking new pixels as they finish; pixels with more than 1024
+ *     records or lists out of depth order are composited by a direct sweep in
+ *     the last launch.  The
  *     image is processed in chunks of pixels whose pieces fit the pool;
  *   VDI_SCHED_LANE (5, k <= 8; larger k take VDI_SCHED_STAGED): a warp copies
  *     the records of 32 consecutive pixels into shared memory with coalesced

@@ -12,13 +12,14 @@
 //     mixture (extinctions add; colour is the extinction-weighted mean), summed
 //     exactly in 128-bit fixed point so that every schedule gets the same bits.
 // The pieces feed the supersegment state machine (Eq. 1) inside the per-pixel
-// bisection search for gamma: a march evaluates the next two bisection levels
-// at once (midpoint and both children) and records, per candidate, the
-// interval of gamma over which all of its decisions repeat; the sequential
-// bisection is replayed from the recorded counts, marching again only for a
-// midpoint no record covers, so the result is that of plain bisection.  The
-// first march also counts non-transparent pieces (the count at gamma = 0).  A
-// final sweep emits at most n_s supersegments into the regular layout with a
+// bisection search for gamma: a march evaluates several midpoints at once and
+// the sequential bisection is replayed from their counts, marching again only
+// for a midpoint without one, so the result is that of plain bisection.  The
+// flat search evaluates the four likeliest midpoints (vdi_search.cuh); the
+// direct sweeps the next two levels (midpoint and both children), recording per
+// candidate the interval of gamma over which all of its decisions repeat, and
+// count the non-transparent pieces (the count at gamma = 0) in their first
+// march.  A final sweep emits at most n_s supersegments into the regular layout with a
 // zero tail.
 //
 // Schedules (the same result, bit for bit; chosen per request by the
@@ -33,8 +34,8 @@
 //     count (list_hist / list_offsets / list_scatter) and
 //     composite_flat_kernel searches and emits them;
 //   VDI_SCHED_STAGED (4): composite_build_kernel builds each pixel's pieces
-//     with the whole warp (coalesced span loads, merge-path sort of the bounds,
-//     exact prefix scan of the mixture terms) into the pool, and
+//     with a warp, or four for long lists (coalesced span loads, merge-path sort
+//     of the bounds, exact prefix scan of the mixture terms) into the pool, and
 //     composite_flat_kernel searches and emits every pixel; the host runs the
 //     pixels in chunks whose pieces fit the pool;
 //   both list pixels they cannot stage (more than 480 / 1024 records, pieces
@@ -44,7 +45,7 @@
 //     lists on every march, heads in registers (1, K <= 8) or in shared memory
 //     under a winner tree (2; 3 with three levels per march).
 // composite_flat_kernel runs the search and the emission as one loop whose
-// body handles one piece of a lane's current march, so lanes at different
+// body handles four pieces of a lane's current march, so lanes at different
 // marches or pixels execute the same instructions; lanes at the end of a
 // march wait for others to end theirs together, and a lane that finishes its
 // pixel takes the next one.
@@ -727,49 +728,7 @@ __device__ __forceinline__ void cq_step(CompCountQ& s, const Piece& x, float g2)
     }
 }
 
-// cq_step written without branches: every outcome
-// is computed with the same rounded operations and selected, so the decisions
-// are bit for bit those of the branchy steps, and a visitor's candidates form
-// straight-line code whose dependency chains interleave.
-struct StepSel {
-    bool fresh, close;
-};
-
-// A step that neither opens S (fresh) nor absorbs into it leaves S closed, and the colour, opacity,
-// optical depth and bounds of a closed S are never read again (the next fresh piece overwrites all of
-// them), so those steps may take the absorbing form as well: one select per value instead of two.
-template <typename S>
-__device__ __forceinline__ void apply_step(S& s, const Piece& x, StepSel d) {
-    const float T = __fsub_rn(1.f, s.A);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) s.P[c] = d.fresh ? x.P[c] : __fmaf_rn(T, x.P[c], s.P[c]);
-    s.A = d.fresh ? x.a : __fmaf_rn(T, x.a, s.A);
-    s.L2 = d.fresh ? x.lgT : __fadd_rn(s.L2, x.lgT);
-    s.fS = d.fresh ? x.f : s.fS;
-    s.bS = x.b;
-    s.open = d.fresh || (s.open && !d.close);
-    s.cnt += d.fresh ? 1 : 0;
-}
-
-template <typename S>
-__device__ __forceinline__ float piece_ratio(const S& s, const Piece& x) {
-    const float lx = __fsub_rn(x.b, x.f), lS = __fsub_rn(s.bS, s.fS);
-    return (lx > 0.f && lS > 0.f) ? __fmul_rn(lx, rcp_approx(lS)) : 1.f;
-}
-
-__device__ __forceinline__ void cq_step_select(CompCountQ& s, const Piece& x, float g2) {
-    float q = 0.f;
-    const bool crit = s.open && criterion_q(s.P, s.A, s.L2, piece_ratio(s, x), x.P, g2, q);
-    s.qhi = crit ? fminf(s.qhi, q) : s.qhi;               // crit implies an open S
-    s.qlo = (s.open && !crit) ? fmaxf(s.qlo, q) : s.qlo;
-    const bool opaque = x.a > 0.f;
-    apply_step(s, x, StepSel{opaque && (!s.open || crit), crit && !opaque});
-}
-
-// SELECT: the branch-free steps (faster where the pieces come from the staged
-// buffer, 2.46 vs 2.76 s at 2048^2, K = 32; slower in the direct sweepers, 8.1
-// vs 7.5 ms on the 512^3 frame, whose piece generation interleaves with them)
-template <int NC, bool SELECT>
+template <int NC>
 struct CountVisitorQ {
     CompCountQ st[NC];
     float g2[NC];
@@ -787,10 +746,7 @@ struct CountVisitorQ {
     __device__ __forceinline__ void operator()(const Piece& x) {
         nt += x.a > 0.f;
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            if constexpr (SELECT) cq_step_select(st[c], x, g2[c]);
-            else cq_step(st[c], x, g2[c]);
-        }
+        for (int c = 0; c < NC; ++c) cq_step(st[c], x, g2[c]);
     }
 };
 
@@ -867,7 +823,6 @@ __device__ __forceinline__ void tree_candidates(float lo, float hi, float g[(1 <
 // memory with P leaves (KMAX == 0, K <= P).
 template <int KMAX, int P, int PREC>
 struct Sweeper {
-    static constexpr bool kSelectSteps = false;  // counting steps with branches (see CountVisitorQ)
     const PeIn* pe;
     int k;
     uint32_t p;
@@ -919,7 +874,7 @@ __device__ __forceinline__ void composite_search_emit(SW& sw, const OutDev& out,
     {
         CountTable t;
         t.n = 0;
-        CountVisitorQ<NC, SW::kSelectSteps> v;
+        CountVisitorQ<NC> v;
         float g[NC];
         v.reset();
         tree_candidates<NLEV>(0.f, 2.f, g);
@@ -1087,8 +1042,8 @@ __device__ __forceinline__ void finish_pixel(const OutDev& out, uint32_t p, int 
 // ---------------------------------------------------------------------------
 // Staged path
 // ---------------------------------------------------------------------------
-// A warp takes 32 consecutive pixels at a time.  Phase G builds the pieces of
-// each of them in turn, the whole warp on one pixel: it loads the pixel's
+// A warp (or a CTA of four, for long lists) takes 32 consecutive pixels at a time.  Phase G builds the pieces of
+// each of them in turn, every thread on one pixel: they load the pixel's
 // records from all K lists, drops those with b <= f, sorts their bounds (each
 // list's bounds are already in order, so a stable merge of the K runs: log2 K
 // rounds in which every bound finds its place in its partner run by binary
@@ -1773,7 +1728,6 @@ __device__ __forceinline__ int sweep_slab(const SLAB& S, int k, const uint32_t s
 // pixels take the sweep.
 template <class SLAB>
 struct SlabSweeper {
-    static constexpr bool kSelectSteps = false;  // counting steps with branches (see CountVisitorQ)
     const SLAB* S;
     int k;
     uint32_t st[kLaneKMax], cnt[kLaneKMax];
@@ -2201,7 +2155,9 @@ __global__ void __launch_bounds__(kStageWarps * 32, VDI_BUILD_MIN_BLOCKS) compos
 // same, bit for bit.  The pieces come from a pool in the workspace (written by
 // the batch pass), one contiguous run per pixel.
 //
-// What bounds it: instructions per piece.  Four candidates run as two packed
+// What bounds it: instructions per piece (640 x 480, K = 32 dense: the search pass's two chunks of 131,072 pixels
+// took 35 ms each with three candidates value by value and a load per piece; the whole call 171 -> 70 ms with the
+// build's changes).  Four candidates run as two packed
 // pairs in the form that takes the fewest operations:
 //   - a closed S is P = A = L2 = 0, and the next non-transparent piece opens a new
 //     one;
@@ -2217,8 +2173,8 @@ __global__ void __launch_bounds__(kStageWarps * 32, VDI_BUILD_MIN_BLOCKS) compos
 #ifndef VDI_FLAT_END_BATCH
 #define VDI_FLAT_END_BATCH 16
 #endif
-// resident CTAs of the flat pass per SM over the dense pieces of the pooled and batched paths (the lane
-// path takes as many as the registers allow)
+// resident CTAs of the flat pass per SM over the dense pieces of the pooled and batched paths: 4 and 5 measured alike
+// (72.5 and 73.0 ms for the dense call), 6 spills (78.5)
 #ifndef VDI_FLAT_CTAS_PER_SM
 #define VDI_FLAT_CTAS_PER_SM 5
 #endif
@@ -2405,9 +2361,8 @@ __device__ __forceinline__ void flat_loop(const SRC& src, const PiecePool& pool,
                     float k0, k1, k2, k3;
                     unpk(st[0].kept, k0, k1);
                     unpk(st[1].kept, k2, k3);
-                    search_end_march(sh, L.nt - (int)k0, L.nt - (int)k1, L.nt - (int)k2, L.nt - (int)k3, L.out->n_s,
-                                     iters, L.nt);
-                    emit = sh.phase == kBisDone;
+                    search_end_march(sh, L.nt - (int)k0, L.nt - (int)k1, L.nt - (int)k2, L.nt - (int)k3, L.out->n_s);
+                    emit = sh.done != 0;
                     count = !emit;
                 }
             }
@@ -2435,8 +2390,7 @@ __device__ __forceinline__ void flat_loop(const SRC& src, const PiecePool& pool,
                             emit = true;
                         } else {
                             if (CENSUS) cs.searched += 1;
-                            // (the distance never reaches 2: one supersegment there)
-                            search_start(sh, L.out->n_s, iters, L.nt, 1, false);
+                            search_start(sh, L.out->n_s, iters, L.nt);
                             count = true;
                         }
                     }
@@ -2667,7 +2621,7 @@ struct BatchEntry {
 
 struct BatchBuildArgs {
     unsigned int* counter;  // item counter
-    uint32_t* list;         // [0] entries, [1] next entry of the flat pass, [2] pool pieces taken; entries from word 8
+    uint32_t* list;         // [0] entries, [1] next entry of the flat pass, [2], [3] pool pieces taken; entries from word 8
     PiecePool pool;
     uint32_t item0, item1;  // the chunk's items
 };
@@ -3071,7 +3025,8 @@ constexpr uint64_t kBatchListCap = 1u << 22;
 constexpr uint64_t kBatchPoolCap = 1u << 28;
 
 static uint64_t batch_pixel_pieces(const ReqDev& r) {
-    const uint64_t est = 2ull * (uint64_t)r.k * (uint64_t)(r.out.n_s > 0 ? r.out.n_s : 1) + 1;
+    // (rounded up to the groups of four that a run takes)
+    const uint64_t est = (2ull * (uint64_t)r.k * (uint64_t)(r.out.n_s > 0 ? r.out.n_s : 1) + 2) / 4 * 4;
     return est < kPoolPiecesPerPixel ? est : kPoolPiecesPerPixel;
 }
 

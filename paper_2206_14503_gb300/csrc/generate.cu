@@ -298,7 +298,7 @@ struct CacheRef {
 // them (up to c->cap).  NC gamma candidates ride along (NC may be 0).  OWNED:
 // PE e's samples under the ownership map of *ga; *runs receives the number of
 // domain runs holding a non-transparent sample (the count at gamma = 2).
-template <int NC, bool OWNED = false>
+template <int NC, bool OWNED = false, int AHEAD = 1>
 __device__ __forceinline__ int first_march(const Ray& r, int k0, int k1, const BrickDev& b, const float4* lut2,
                                            float scale255, const float* g2, int cap, const CacheRef* c, int* cnt,
                                            Census& cs, const GenReq* ga = nullptr, int e = 0, int* runs = nullptr,
@@ -337,7 +337,7 @@ __device__ __forceinline__ int first_march(const Ray& r, int k0, int k1, const B
         });
         *runs = nruns;
     } else {
-        march(r, k0, k1, b, lut2, scale255, visit);
+        march<AHEAD>(r, k0, k1, b, lut2, scale255, visit);
     }
 #pragma unroll
     for (int q = 0; q < NC; ++q) cnt[q] = st[q].cnt;
@@ -580,11 +580,19 @@ __device__ __forceinline__ float bisect_gamma(const Ray& r, int k0, int k1, cons
 // march is inlined: out-of-line calls in this persistent loop cost far more
 // than the spills inlining brings (the learned choice took 80.6 ms with the
 // refinement, its marches and the search fallback out of line, 65.6 ms inlined).
-template <bool LEARNED, bool OWNED>
+// samples on the way in the first march: the fixed-gamma kernel has the registers for two, the others do not
+#ifndef VDI_FIXED_AHEAD
+#define VDI_FIXED_AHEAD 2
+#endif
+#ifndef VDI_LEARNED_AHEAD
+#define VDI_LEARNED_AHEAD 1
+#endif
+template <bool LEARNED, bool OWNED, bool FIXED>
 __device__ __forceinline__ void count_ray(const GenReq& a, const BrickDev& b, const CompactDev& o, int e, int i, int j,
                                           const float4* __restrict__ lut2, const CacheRef& cref, Census& cs,
                                           unsigned long long& rays, uint2* rng) {
-    const int mode = LEARNED ? 3 : a.mode;
+    constexpr int kAhead = FIXED ? VDI_FIXED_AHEAD : (LEARNED ? VDI_LEARNED_AHEAD : 1);
+    const int mode = FIXED ? 0 : (LEARNED ? 3 : a.mode);
     const size_t p = (size_t)j * a.cam.W + i;
     Ray r;
     int k0 = 0, k1 = 0;
@@ -601,7 +609,7 @@ __device__ __forceinline__ void count_ray(const GenReq& a, const BrickDev& b, co
         if (mode == 0) {
             const float g2[1] = {__fmul_rn(a.gamma, a.gamma)};
             int c[1];
-            const int nt = first_march<1, OWNED>(r, k0, k1, b, lut2, a.scale255, g2, a.n_s, nullptr, c, cs, &a, e,
+            const int nt = first_march<1, OWNED, kAhead>(r, k0, k1, b, lut2, a.scale255, g2, a.n_s, nullptr, c, cs, &a, e,
                                                  &runs, ks);
             count = c[0];
             if (!OWNED && rng && nt > 0) *rng = make_uint2((unsigned)kspan[0], (unsigned)kspan[1]);
@@ -614,7 +622,7 @@ __device__ __forceinline__ void count_ray(const GenReq& a, const BrickDev& b, co
                 // one march: count at the given gamma, non-transparent count, cache
                 const float g2[1] = {__fmul_rn(gamma, gamma)};
                 int c[1];
-                nt = first_march<1, OWNED>(r, k0, k1, b, lut2, a.scale255, g2, INT_MAX, use_cache ? &cref : nullptr,
+                nt = first_march<1, OWNED, kAhead>(r, k0, k1, b, lut2, a.scale255, g2, INT_MAX, use_cache ? &cref : nullptr,
                                            c, cs, &a, e, &runs, ks);
                 cp = c[0];
                 if (mode == 2) {
@@ -672,8 +680,15 @@ __device__ __forceinline__ void census_flush_gen(const Census& cs, unsigned long
 #ifndef VDI_LEARNED_MIN_BLOCKS
 #define VDI_LEARNED_MIN_BLOCKS 10
 #endif
-template <bool CENSUS, bool LEARNED, bool OWNED = false>
-__global__ void __launch_bounds__(kCountThreads, LEARNED ? VDI_LEARNED_MIN_BLOCKS : VDI_COUNT_MIN_BLOCKS)
+// and the fixed-gamma one's: one march a ray and no search, so it needs no spills, takes more resident warps and
+// has the cells of two samples on the way.  384^3, K = 1, 1280 x 720: generation 3.20 -> 2.65 ms against the search
+// kernel's march (16 blocks spill: 4.6 ms; 12: 3.09 on the host where 14 took 3.06)
+#ifndef VDI_FIXED_MIN_BLOCKS
+#define VDI_FIXED_MIN_BLOCKS 14
+#endif
+template <bool CENSUS, bool LEARNED, bool OWNED = false, bool FIXED = false>
+__global__ void __launch_bounds__(kCountThreads, FIXED ? VDI_FIXED_MIN_BLOCKS
+                                                       : (LEARNED ? VDI_LEARNED_MIN_BLOCKS : VDI_COUNT_MIN_BLOCKS))
     gen_count_kernel(
     const __grid_constant__ GenArgs a) {
     __shared__ float4 lut2[2 * 257];
@@ -699,13 +714,19 @@ __global__ void __launch_bounds__(kCountThreads, LEARNED ? VDI_LEARNED_MIN_BLOCK
         int i, j;
         tile_pixel(a.r.tiles_x, (int)(item % tiles), kCountTileH, i, j);
         if (i >= a.r.cam.W || j >= a.r.cam.H) continue;
-        count_ray<LEARNED, OWNED>(a.r, a.b[e], a.out[e], e, i, j, lut2, cref, cs, rays,
+        count_ray<LEARNED, OWNED, FIXED>(a.r, a.b[e], a.out[e], e, i, j, lut2, cref, cs, rays,
                                   a.ranges ? a.ranges + (size_t)e * a.r.cam.W * a.r.cam.H +
                                                  ((size_t)j * a.r.cam.W + i)
                                            : nullptr);
     }
     if (CENSUS) census_flush_gen(cs, rays, a.status);
 }
+
+// samples on the way in the emission's march, and its block bound: 7 blocks hold two without spills (64^3 frame,
+// whose 200 samples a ray are one latency after the other: 300 -> 293 us)
+#ifndef VDI_EMIT_AHEAD
+#define VDI_EMIT_AHEAD 2
+#endif
 
 struct RecOut {
     float f, b, P[3], A;
@@ -821,7 +842,7 @@ __device__ __forceinline__ void emit_ray(const GenReq& a, const BrickDev& b, con
             st.m = 0.f;
         });
     } else {
-        march(r, k0, k1, b, lut2, a.scale255, visit);
+        march<VDI_EMIT_AHEAD>(r, k0, k1, b, lut2, a.scale255, visit);
     }
     if (st.m != 0.f) {
         if (written < room) {
@@ -837,7 +858,7 @@ __device__ __forceinline__ void emit_ray(const GenReq& a, const BrickDev& b, con
 
 template <bool OWNED, bool REGULAR>
 #ifndef VDI_EMIT_MIN_BLOCKS
-#define VDI_EMIT_MIN_BLOCKS 8
+#define VDI_EMIT_MIN_BLOCKS 7
 #endif
 __global__ void __launch_bounds__(kEmitThreads, VDI_EMIT_MIN_BLOCKS) gen_emit_kernel(const __grid_constant__ GenArgs a) {
     __shared__ float4 lut2[2 * 257];
@@ -869,12 +890,14 @@ struct GenBatchReq {
 struct GenBatchPe {
     BrickDev b;
     CompactDev out;
+    uint64_t ray_begin;  // (PE, pixel) pairs of the PEs before it
 };
 
 struct GenBatchHeader {
     uint32_t n, total_items, total_eitems, total_pes;
     uint32_t total_chunks, pad;
     uint64_t reqs_off, pes_off, lists_off;
+    uint64_t total_rays;  // (PE, pixel) pairs
 };
 
 struct GenBatchArgs {
@@ -886,6 +909,7 @@ struct GenBatchArgs {
     unsigned int* counter;
     float2* cache;
     int cache_cap, slots;
+    uint2* ranges;  // each (PE, pixel)'s span, as GenArgs::ranges (nullptr: the workspace has no room for them)
 };
 
 // the request holding work item `item` (the last one beginning at or before it)
@@ -931,7 +955,8 @@ __global__ void __launch_bounds__(kCountThreads, VDI_COUNT_MIN_BLOCKS) gen_count
         tile_pixel(br.r.tiles_x, (int)(local % tiles), kCountTileH, i, j);
         if (i >= br.r.cam.W || j >= br.r.cam.H) continue;
         const GenBatchPe& pe = a.pes[br.pe_begin + e];
-        count_ray<false, false>(br.r, pe.b, pe.out, e, i, j, lut2, cref, cs, rays, nullptr);
+        count_ray<false, false, false>(br.r, pe.b, pe.out, e, i, j, lut2, cref, cs, rays,
+                                       a.ranges ? a.ranges + pe.ray_begin + ((size_t)j * br.r.cam.W + i) : nullptr);
     }
 }
 
@@ -947,7 +972,8 @@ __global__ void __launch_bounds__(kEmitThreads, VDI_EMIT_MIN_BLOCKS) gen_emit_ba
     tile_pixel(br.r.tiles_x, (int)(local % etiles), kEmitTileH, i, j);
     const bool inside = i < br.r.cam.W && j < br.r.cam.H;
     const GenBatchPe& pe = a.pes[br.pe_begin + e];
-    emit_ray<false, false>(br.r, pe.b, pe.out, e, i, j, inside, lut2, a.status, nullptr);
+    emit_ray<false, false>(br.r, pe.b, pe.out, e, i, j, inside, lut2, a.status,
+                           a.ranges ? a.ranges + pe.ray_begin : nullptr);
 }
 
 static void fill_req(GenReq& r, int k, const float* lut, const CamDev& cam, const int dims[3], float scale255,
@@ -1101,7 +1127,19 @@ vdi_status launch_gen_count(const BrickDev* bricks, int k, const float* lut, con
     else if (a.r.own.map) gen_count_kernel<false, false, true><<<ctas, kCountThreads, 0, st>>>(a);
     else if (census && learned) gen_count_kernel<true, true><<<ctas, kCountThreads, 0, st>>>(a);
     else if (census) gen_count_kernel<true, false><<<ctas, kCountThreads, 0, st>>>(a);
-    else if (learned) gen_count_kernel<false, true><<<ctas, kCountThreads, 0, st>>>(a);
+    else if (a.r.mode == 0) {
+        // (its own grid: it takes no slots of the cache)
+        int dev = 0, sms = 0, per_sm = 0;
+        s = cuda_check(cudaGetDevice(&dev), "cudaGetDevice");
+        if (s == VDI_OK) s = cuda_check(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
+        if (s == VDI_OK)
+            s = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                               &per_sm, gen_count_kernel<false, false, false, true>, kCountThreads, 0),
+                           "occupancy");
+        if (s != VDI_OK) return s;
+        const unsigned most = (unsigned)(sms * (per_sm > 0 ? per_sm : 1));
+        gen_count_kernel<false, false, false, true><<<most < items ? most : items, kCountThreads, 0, st>>>(a);
+    } else if (learned) gen_count_kernel<false, true><<<ctas, kCountThreads, 0, st>>>(a);
     else gen_count_kernel<false, false><<<ctas, kCountThreads, 0, st>>>(a);
     return cuda_check(cudaGetLastError(), "gen_count_kernel launch");
 }
@@ -1150,7 +1188,7 @@ vdi_status gen_batch_table_pack(const vdi_gen_request* reqs, int n, const vdi_pa
     GenBatchReq* rd = reinterpret_cast<GenBatchReq*>(base + hd->reqs_off);
     GenBatchPe* pd = reinterpret_cast<GenBatchPe*>(base + hd->pes_off);
     ScanList* ld = reinterpret_cast<ScanList*>(base + hd->lists_off);
-    uint64_t items = 0, eitems = 0, chunks = 0;
+    uint64_t items = 0, eitems = 0, chunks = 0, rays = 0;
     uint32_t pe = 0;
     for (int q = 0; q < n; ++q) {
         const vdi_gen_request& g = reqs[q];
@@ -1173,6 +1211,8 @@ vdi_status gen_batch_table_pack(const vdi_gen_request* reqs, int n, const vdi_pa
             pd[pe].b = brick_dev(g.bricks[e]);
             const vdi_compact& o = g.out[e];
             pd[pe].out = CompactDev{o.counts, o.offsets, o.rgba, o.fb, o.gamma, o.capacity};
+            pd[pe].ray_begin = rays;
+            rays += (uint64_t)npix;
             ld[pe].counts = o.counts;
             ld[pe].offsets = o.offsets;
             ld[pe].n = npix;
@@ -1187,18 +1227,20 @@ vdi_status gen_batch_table_pack(const vdi_gen_request* reqs, int n, const vdi_pa
     hd->total_eitems = (uint32_t)eitems;
     hd->total_pes = pe;
     hd->total_chunks = (uint32_t)chunks;
+    hd->total_rays = rays;
     hd->pad = 0;
     return VDI_OK;
 }
 
 // [0, 256) status header, [256, 512) work counter, the prefix sum's partial
-// sums, then (optionally) the sample cache
+// sums, then (optionally) the sample cache and, after it, every (PE, ray)'s span
 size_t gen_batched_workspace_bytes(const void* host_table) {
     const GenBatchHeader* hd = static_cast<const GenBatchHeader*>(host_table);
     int ctas = 0;
     size_t cache = 0;
     if (gen_count_grid(ctas) == VDI_OK) cache = gen_cache_bytes(ctas);
-    return kGenFixed + align_up((size_t)hd->total_chunks * sizeof(uint64_t), 256) + align_up(cache, 256);
+    return kGenFixed + align_up((size_t)hd->total_chunks * sizeof(uint64_t), 256) + align_up(cache, 256) +
+           (cache > 0 ? align_up((size_t)hd->total_rays * sizeof(uint2), 256) : 0);
 }
 
 vdi_status launch_gen_batched(const void* dev_table, const void* host_table, void* workspace, size_t ws_bytes,
@@ -1229,6 +1271,10 @@ vdi_status launch_gen_batched(const void* dev_table, const void* host_table, voi
         a.cache_cap = kCacheCap;
         a.cache = reinterpret_cast<float2*>(ws + fixed);
     }
+    a.ranges = nullptr;
+    const size_t spans = fixed + align_up(gen_cache_bytes(ctas), 256);
+    if (a.cache && ws_bytes >= spans + (size_t)hd->total_rays * sizeof(uint2))
+        a.ranges = reinterpret_cast<uint2*>(ws + spans);
     if ((unsigned)ctas > hd->total_items) ctas = (int)hd->total_items;
     gen_count_batched_kernel<<<ctas, kCountThreads, 0, st>>>(a);
     s = cuda_check(cudaGetLastError(), "gen_count_batched_kernel launch");

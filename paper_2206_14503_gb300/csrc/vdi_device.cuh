@@ -365,27 +365,41 @@ __device__ __forceinline__ void sample_from(float w0, float w1, float w2, const 
 }
 
 // March over samples [k0, k1) of ray r in brick b, calling f(k, sample) in
-// order.  The next sample's cell is loaded while the current one is
-// processed, so the load latency overlaps the state-machine work.
-template <typename F>
+// order.  The cell of the sample AHEAD samples on is loaded while the current
+// one is processed, so the load latency overlaps the state-machine work.  A cell
+// is 32 bytes of its own for most samples of a large volume, and a kernel with
+// registers to spare hides more of its latency with several on the way: each
+// sample ahead takes 11 registers, and a kernel that spills for them loses more
+// (512^3 frame with 2 in the search kernel: 28.4 -> 29.4 ms).
+template <int AHEAD, typename F>
 __device__ __forceinline__ void march(const Ray& r, int k0, int k1, const BrickDev& b, const float4* __restrict__ lut2,
                                       float scale255, F&& f) {
-    long long P[3];
+    long long P[3];  // the next sample to load
 #pragma unroll
     for (int a = 0; a < 3; ++a) P[a] = r.P0[a] + (long long)k0 * r.D[a];
-    float4 clo, chi;
-    cell_load(P, b, clo, chi);
-    for (int k = k0; k < k1; ++k) {
-        const float w0 = fixed_frac(P[0]), w1 = fixed_frac(P[1]), w2 = fixed_frac(P[2]);
+    float4 lo[AHEAD], hi[AHEAD];
+    float w[AHEAD][3];
+    auto load = [&](int u) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) w[u][a] = fixed_frac(P[a]);
+        cell_load(P, b, lo[u], hi[u]);
 #pragma unroll
         for (int a = 0; a < 3; ++a) P[a] += r.D[a];
-        float4 nlo, nhi;
-        cell_load(P, b, nlo, nhi);  // next sample's cell, in flight during this sample's work
-        Sample s;
-        sample_from(w0, w1, w2, clo, chi, lut2, scale255, s);
-        f(k, s);
-        clo = nlo;
-        chi = nhi;
+    };
+#pragma unroll
+    for (int u = 0; u < AHEAD; ++u) load(u);
+    for (int k = k0; k < k1; k += AHEAD) {
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {
+            if (k + u < k1) {
+                const float w0 = w[u][0], w1 = w[u][1], w2 = w[u][2];
+                const float4 clo = lo[u], chi = hi[u];
+                load(u);
+                Sample s;
+                sample_from(w0, w1, w2, clo, chi, lut2, scale255, s);
+                f(k + u, s);
+            }
+        }
     }
 }
 
