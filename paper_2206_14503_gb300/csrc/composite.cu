@@ -1999,8 +1999,11 @@ constexpr size_t lane_smem_bytes() {
     return kLaneWarps * sizeof(LaneSlab<PREC, CAP>);
 }
 
+// Four CTAs per SM, as many as their slabs (46 KB each) allow: the sweeps' serial chains want every warp, and a
+// kernel of 136 registers kept three (320 x 240, FP16 records: K = 4, N_S = 12 dense 4.64 -> 3.30 ms with four,
+// K = 2, N_S = 32 dense 5.76 -> 4.02).
 template <int PREC, bool CENSUS>
-__global__ void __launch_bounds__(kLaneWarps * 32) composite_lane_kernel(const __grid_constant__ CompArgs a,
+__global__ void __launch_bounds__(kLaneWarps * 32, 4) composite_lane_kernel(const __grid_constant__ CompArgs a,
                                                                         const __grid_constant__ LaneArgs la) {
     using Slab = LaneSlab<PREC, kLaneRCap>;
     extern __shared__ __align__(16) unsigned char lane_smem[];
