@@ -162,13 +162,29 @@ __device__ __forceinline__ void u128_add_signed(U128& s, const U128& x, unsigned
         : "l"(x.lo ^ neg), "l"(x.hi ^ neg), "l"(neg));
 }
 
-// The conversions between FP32 and this format in 32-bit integer operations: the hardware's conversions to and from
-// 64-bit integers run on the FP64 pipe, 2 lanes an SM on this chip (16 cycles a warp for each, 8 of them per bound
-// and per piece: more than half of the pooled build's time).
-
-// v in [0, 2^56] as fixed point: the significand shifted to its place, exact for v >= 2^-41 (its 24 bits fit the
-// 64 fraction bits), truncated below
+// The conversions between FP32 and this format, v in [0, 2^56] as fixed point: exact for v >= 2^-41 (the 24-bit
+// significand fits the 64 fraction bits), truncated below.
 __device__ __forceinline__ U128 to_fixed(float v) {
+    const float ip = truncf(v);
+    U128 r;
+    r.hi = __float2ull_rz(ip);
+    r.lo = __float2ull_rz(__fmul_rn(__fsub_rn(v, ip), 18446744073709551616.f));
+    return r;
+}
+
+__device__ __forceinline__ float from_fixed(const U128& s) {
+    return __fmaf_rn(__ull2float_rn(s.lo), 5.421010862427522e-20f, __ull2float_rn(s.hi));
+}
+
+// The same conversions (the same bits) in 32-bit integer operations, for the pooled build, whose warps are full: the
+// hardware's conversions to and from 64-bit integers run on the FP64 pipe, 2 lanes an SM on this chip (16 cycles a
+// warp for each, 8 of them per bound and per piece: more than half of the pooled build's time).  The sweeps keep the
+// hardware's: they convert in code of its own for each of up to eight heads, with few lanes at work, and the integer
+// form makes that code several times as long (320 x 240, K = 8, lane schedule: N_S = 32 dense 264 ms with the integer
+// form, 122 with the hardware's; N_S = 4 ragged 1.68 and 1.32; N_S = 12 dense 14.1 and 16.5).
+
+// the significand shifted to its place
+__device__ __forceinline__ U128 to_fixed_int(float v) {
     const uint32_t bits = __float_as_uint(v);
     const int sh = (int)(bits >> 23) - 86;  // of the significand's last bit, from the last fraction bit
     const uint32_t m = (bits & 0x7FFFFFu) | 0x800000u;
@@ -192,7 +208,7 @@ __device__ __forceinline__ float u64_to_float(unsigned long long x) {
     return __fmul_rn(__uint2float_rn(top | sticky), __uint_as_float((uint32_t)(159 - z) << 23));  // 2^(32 - z)
 }
 
-__device__ __forceinline__ float from_fixed(const U128& s) {
+__device__ __forceinline__ float from_fixed_int(const U128& s) {
     return __fmaf_rn(u64_to_float(s.lo), 5.421010862427522e-20f, u64_to_float(s.hi));
 }
 
@@ -259,10 +275,10 @@ __device__ __forceinline__ Contrib contrib_of(const float4& t) {
     const bool op = OPQ && t.w < 0.f;
     r.op = op ? 1 : 0;
     const float v[3] = {t.x, t.y, t.z};
-    r.M = to_fixed(op ? 0.f : t.w);
+    r.M = to_fixed_int(op ? 0.f : t.w);
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-        const U128 x = to_fixed(v[q]);
+        const U128 x = to_fixed_int(v[q]);
         u128_zero(r.MC[q]);
         u128_zero(r.OC[q]);
         if (op) r.OC[q] = x;
@@ -313,8 +329,11 @@ __device__ __forceinline__ void sums_update(MixSums& m, const Contrib& x) {
 
 // The piece [t, t1] of an active set with sums m; `whole` when exactly one
 // record is active and it spans [t, t1] (its colour and opacity are wc).
+// INT: with the integer conversion.
+template <bool INT = false>
 __device__ __forceinline__ void piece_from(const MixSums& m, bool whole, const RecC& wr, float t, float t1,
                                            Piece& x) {
+    const auto value = [](const U128& v) { return INT ? from_fixed_int(v) : from_fixed(v); };
     x.f = t;
     x.b = t1;
     if (whole) {
@@ -331,18 +350,18 @@ __device__ __forceinline__ void piece_from(const MixSums& m, bool whole, const R
         const float inv = 1.f / (float)m.nop;
         x.a = 1.f;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) x.P[q] = __fmul_rn(from_fixed(m.OC[q]), inv);
+        for (int q = 0; q < 3; ++q) x.P[q] = __fmul_rn(value(m.OC[q]), inv);
         x.lgT = -INFINITY;
         return;
     }
-    const float M = m.nact > 0 ? from_fixed(m.M) : 0.f;
+    const float M = m.nact > 0 ? value(m.M) : 0.f;
     if (M > 0.f) {
         // emission-absorption mixture (Eq. 2 when one record covers the piece in part)
         x.lgT = -__fmul_rn(M, __fsub_rn(t1, t));
         x.a = __fsub_rn(1.f, ex2_approx(x.lgT));
         const float s = __fmul_rn(x.a, rcp_approx(M));
 #pragma unroll
-        for (int q = 0; q < 3; ++q) x.P[q] = __fmul_rn(from_fixed(m.MC[q]), s);
+        for (int q = 0; q < 3; ++q) x.P[q] = __fmul_rn(value(m.MC[q]), s);
     } else {
         // a gap, or only fully transparent records
         x.P[0] = x.P[1] = x.P[2] = 0.f;
@@ -1291,7 +1310,7 @@ __device__ __forceinline__ bool stage_scan(const PeIn* pe, StageSmem<RMAX>& S, S
             }
         }
         Piece x;
-        piece_from(st.s, whole, wc, t, t1, x);
+        piece_from<true>(st.s, whole, wc, t, t1, x);
         const size_t at = out.at(row);
         out.A[at] = make_float4(x.P[0], x.P[1], x.P[2], x.a);
         out.B[at] = make_float2(x.b, x.lgT);
