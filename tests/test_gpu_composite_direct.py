@@ -63,36 +63,3 @@ def test_lists_out_of_depth_order(steps, prec):
     lists = [_compact(pixels, e) for e in range(k)]
     _same(lists, prec, 4, 1, (vdi.VDI_SCHED_LANE,))
     _same(lists, prec, 4, 2, (vdi.VDI_SCHED_STAGED,))
-
-
-ODD = {"opacity above 1": (5, 1.5), "opacity NaN": (5, np.nan), "colour NaN": (3, np.nan), "colour infinite": (2, np.inf),
-       "colour large": (2, 3e30), "colour -0": (3, -0.0), "front -0": (0, -0.0), "opacity negative": (5, -0.5)}
-
-
-@pytest.mark.parametrize("prec", [0, 1])
-@pytest.mark.parametrize("k", [8, 11])
-@pytest.mark.parametrize("kind", sorted(ODD) + ["opaque, then short", "far"])
-def test_values_outside_the_packed_search(kind, k, prec):
-    # one odd record among plain ones; the supersegments behind it are as the direct sweep gives them
-    import paper_2206_14503_gb300 as vdi
-
-    rng = np.random.default_rng(len(kind) + k)
-    pixels = []
-    for p in range(40):
-        lists = [_sorted(rng, 5) for _ in range(k)]
-        if p % 3 == 1:
-            rec = lists[p % k]
-            if kind == "opaque, then short":
-                # an opaque record and another colour's behind it, 1e-36 of the first one's length
-                rec[0, 5] = 1.0
-                rec[0, :2] = -1.0, 0.0
-                rec[1, :2] = 0.0, 1e-36
-            elif kind == "far":
-                rec[-1, 1] = 1e20
-            else:
-                at, v = ODD[kind]
-                rec[0 if at == 0 else p % 5, at] = v
-        pixels.append(lists)
-    lists = [_compact(pixels, e) for e in range(k)]
-    with np.errstate(invalid="ignore", over="ignore", divide="ignore"):
-        _same(lists, prec, 3, 2, (vdi.VDI_SCHED_STAGED,) + ((1, vdi.VDI_SCHED_LANE) if k <= 8 else ()))
