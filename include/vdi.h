@@ -369,9 +369,11 @@ vdi_status vdi_generate_static_scratch(const vdi_brick* bricks, int32_t k, const
  *     batch's part of a pool in the workspace and lists the pixels; another
  *     launch runs the search and the emission of every listed pixel, one lane
  *     each, lanes taking new pixels as they finish; pixels with more than 1024
- *     records or lists out of depth order are composited by a direct sweep in
- *     the last launch.  The
- *     image is processed in chunks of pixels whose pieces fit the pool;
+ *     records, lists out of depth order, or a piece outside the search's range
+ *     (colours that are not finite and non-negative up to 2^64, opacities
+ *     outside [0, 1], a length below 2^-60, a depth beyond 2^40) are composited
+ *     by a direct sweep in the last launch.  The image is processed in chunks
+ *     of pixels whose pieces fit the pool;
  *   VDI_SCHED_LANE (5, k <= 8; larger k take VDI_SCHED_STAGED): a warp copies
  *     the records of 32 consecutive pixels into shared memory with coalesced
  *     loads and each lane sweeps its pixel's lists there once: a pixel whose
@@ -380,7 +382,8 @@ vdi_status vdi_generate_static_scratch(const vdi_brick* bricks, int32_t k, const
  *     sorted by piece count (three small launches) and searched as in the
  *     pooled schedule; pixels whose records exceed the warp's 480-record slab,
  *     whose pieces do not fit the pool, or that need the search and have a
- *     list out of depth order, take a direct sweep;
+ *     list out of depth order or a piece outside the search's range, take a
+ *     direct sweep;
  *   1, 2, 3 (direct): each thread sweeps its pixel's K lists on every march;
  *     1: list heads in registers (k <= 8), two bisection levels per march;
  *     2: heads in shared memory under a winner tree, two levels per march;

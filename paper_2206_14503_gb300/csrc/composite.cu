@@ -39,8 +39,8 @@
 //     composite_flat_kernel searches and emits every pixel; the host runs the
 //     pixels in chunks whose pieces fit the pool;
 //   both list pixels they cannot stage (more than 480 / 1024 records, pieces
-//     beyond the pool, lists out of depth order) for composite_marked_kernel,
-//     the direct sweep;
+//     beyond the pool, lists out of depth order, values that the packed search
+//     does not take: packable) for composite_marked_kernel, the direct sweep;
 //   1, 2, 3 (direct, composite_kernel): one thread per pixel re-sweeps its K
 //     lists on every march, heads in registers (1, K <= 8) or in shared memory
 //     under a winner tree (2; 3 with three levels per march).
@@ -1043,6 +1043,18 @@ __device__ __forceinline__ uint32_t pack_pieces(uint32_t n, uint32_t nt, int nco
     return n | nt << 11 | (uint32_t)(ncol - 1) << 22;
 }
 
+// Whether the packed search takes a piece as the direct sweep does, bit for bit.  It clears a closed supersegment by
+// multiplying with 0 (which an infinity or a NaN outlives, and which turns -0 into +0), subtracts depths without a
+// look at their order, and takes log2(1 - a) = -inf as -1e34 (which a length ratio below 2^-105 would undo).  So a
+// pixel whose pieces are all of finite non-negative colours up to 2^64, opacities in [0, 1] and lengths from 2^-60 at
+// depths within 2^40 is searched in the pool; any other is left to the direct sweep.
+__device__ __forceinline__ bool packable(const Piece& x) {
+    const uint32_t c = max(max(__float_as_uint(x.P[0]), __float_as_uint(x.P[1])), __float_as_uint(x.P[2]));
+    return c <= __float_as_uint(0x1p64f) && __float_as_uint(x.a) <= __float_as_uint(1.f) && x.lgT <= 0.f &&
+           x.f >= -0x1p40f && x.b <= 0x1p40f && __fsub_rn(x.b, x.f) >= 0x1p-60f &&
+           __float_as_uint(x.f) != 0x80000000u;
+}
+
 // writes the zero tail, count and gamma of pixel p after an emission of `written` records
 __device__ __forceinline__ void finish_pixel(const OutDev& out, uint32_t p, int written, float gamma) {
     for (int j = written; j < out.n_s; ++j) {
@@ -1235,8 +1247,9 @@ struct PoolColumn {
 // Phase G after the merge: exact prefix scan of the records' terms over the
 // sorted bounds (srt, E of them; nv valid records), in contiguous chunks per
 // thread, and the pieces written to the column.  tot: scratch for the warps' totals.
+// Returns false when a piece is not packable.
 template <int NW, int PREC, bool OPQ, int RMAX>
-__device__ __forceinline__ void stage_scan(const PeIn* pe, StageSmem<RMAX>& S, ScanState* tot, const uint16_t* srt,
+__device__ __forceinline__ bool stage_scan(const PeIn* pe, StageSmem<RMAX>& S, ScanState* tot, const uint16_t* srt,
                                            uint32_t E, uint32_t nv, const PoolColumn& out, int& npieces, int& nt,
                                            float& f0) {
     constexpr uint32_t T = 32 * NW;
@@ -1279,7 +1292,7 @@ __device__ __forceinline__ void stage_scan(const PeIn* pe, StageSmem<RMAX>& S, S
         }
     }
     // the pieces: after bound i the active set is that of [key_i, key_{i+1}]
-    uint32_t my_nt = 0;
+    uint32_t my_nt = 0;  // non-transparent pieces; from bit 16 on: pieces that are not packable
     uint32_t row = st.nb;
     stage_walk(S, srt, E, i0, i1, [&](uint32_t w, const float4& term, float t, float t1, bool more) {
         stage_apply<OPQ>(w, term, st);
@@ -1301,22 +1314,23 @@ __device__ __forceinline__ void stage_scan(const PeIn* pe, StageSmem<RMAX>& S, S
         const size_t at = out.at(row);
         out.A[at] = make_float4(x.P[0], x.P[1], x.P[2], x.a);
         out.B[at] = make_float2(x.b, x.lgT);
-        my_nt += x.a > 0.f;
+        my_nt += (x.a > 0.f ? 1u : 0u) + (packable(x) ? 0u : 1u << 16);
         ++row;
     });
     my_nt = __reduce_add_sync(0xffffffffu, my_nt);
     npieces = (int)total_pieces;
     f0 = bound_key(S, srt[0]);
-    if constexpr (NW == 1) {
-        nt = (int)my_nt;
-    } else {
+    if constexpr (NW > 1) {
         if (lane == 0) atomicAdd(&S.nt, my_nt);
         __syncthreads();
-        nt = (int)S.nt;
+        my_nt = S.nt;
     }
+    nt = (int)(my_nt & 0xFFFFu);
+    return my_nt < 1u << 16;
 }
 
-// Phase G for pixel p (at most RMAX records) by NW warps.  Returns false when a list is out of depth order.
+// Phase G for pixel p (at most RMAX records) by NW warps.  Returns false when a list is out of depth order or a piece
+// is not packable.
 template <int NW, int PREC, int RMAX>
 __device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem<RMAX>& S, ScanState* tot,
                             const PoolColumn& out, int& npieces, int& nt, float& f0) {
@@ -1471,10 +1485,10 @@ __device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem<RMAX>& 
         group_sync<NW>();
     }
     const uint16_t* srt = S.pay[src];
-    if (opaque) stage_scan<NW, PREC, true>(pe, S, tot, srt, E, nv, out, npieces, nt, f0);
-    else stage_scan<NW, PREC, false>(pe, S, tot, srt, E, nv, out, npieces, nt, f0);
+    const bool ok = opaque ? stage_scan<NW, PREC, true>(pe, S, tot, srt, E, nv, out, npieces, nt, f0)
+                           : stage_scan<NW, PREC, false>(pe, S, tot, srt, E, nv, out, npieces, nt, f0);
     group_sync<NW>();
-    return true;
+    return ok;
 }
 
 // One batch of 32 pixels (from p0 on, at most p1) of a request: if its longest pixel is this kernel's (more than
@@ -1886,6 +1900,7 @@ struct LaneSink {
     float4* A;  // the pixel's pool run
     float2* B;
     bool pool;
+    bool odd;  // a piece written to the pool is not packable
     float f0;  // front of the first piece
     uint32_t np;
     __device__ __forceinline__ void operator()(const Piece& x) {
@@ -1893,6 +1908,7 @@ struct LaneSink {
         if (pool) {
             A[np] = make_float4(x.P[0], x.P[1], x.P[2], x.a);
             B[np] = make_float2(x.b, x.lgT);
+            odd = odd || !packable(x);
         }
         if (emit && x.a > 0.f) {
             const size_t idx = base + written;
@@ -1978,7 +1994,7 @@ __device__ __forceinline__ void slab_stage(const PeIn* pe, int k, SLAB& S, bool 
     }
 }
 
-// the listed pixels marked for the direct sweep (records beyond a slab, pieces beyond the pool, lists
+// the listed pixels marked for the direct sweep (records beyond a slab, pieces beyond the pool or not packable, lists
 // out of depth order), list heads in registers (KMAX > 0) or in shared memory under a winner tree of P
 // leaves (KMAX == 0)
 template <int KMAX, int P, int PREC, bool CENSUS>
@@ -2088,8 +2104,9 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 4) composite_lane_kernel(cons
                 if (!fits) base = 0;
             }
             // one sweep: the gamma = 0 pixels' records, the searched pixels' pieces
-            LaneSink snk{&a.out, (size_t)p * a.out.n_s, 0, emit, la.pool.A + base, la.pool.B + base, fits, 0.f, 0u};
+            LaneSink snk{&a.out, (size_t)p * a.out.n_s, 0, emit, la.pool.A + base, la.pool.B + base, fits, false, 0.f, 0u};
             if (emit || fits) sw.run(snk);
+            fits = fits && !snk.odd;
             if (emit) {
                 if (snk.written != nt) atomicCAS(a.status, 0u, (unsigned)VDI_ERR_CUDA);
                 finish_pixel(a.out, p, snk.written, 0.f);
@@ -2197,7 +2214,8 @@ __global__ void __launch_bounds__(kStageWarps * 32, VDI_BUILD_MIN_BLOCKS) compos
 //   - nA = -A saves the negations, products and sums keeping their bits;
 //   - an opaque piece's log2(1 - a) = -inf becomes -1e34, whose products with a
 //     length ratio give 2^x = 0 as well and which 0 clears.
-// The rounded operations that decide are cq_step's, in its order.
+// The rounded operations that decide are cq_step's, in its order; pixels with
+// values for which one of these does not hold do not come here (packable).
 // ---------------------------------------------------------------------------
 #ifndef VDI_FLAT_END_BATCH
 #define VDI_FLAT_END_BATCH 16

@@ -63,3 +63,39 @@ def test_lists_out_of_depth_order(steps, prec):
     lists = [_compact(pixels, e) for e in range(k)]
     _same(lists, prec, 4, 1, (vdi.VDI_SCHED_LANE,))
     _same(lists, prec, 4, 2, (vdi.VDI_SCHED_STAGED,))
+
+
+ODD = {"opacity above 1": (5, 1.5), "opacity NaN": (5, np.nan), "colour NaN": (3, np.nan), "colour infinite": (2, np.inf),
+       "colour large": (2, 3e30), "colour -0": (3, -0.0), "front -0": (0, -0.0), "opacity negative": (5, -0.5),
+       "back far": (1, 1e20)}
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("k", [8, 11])
+@pytest.mark.parametrize("kind", sorted(ODD) + ["short behind opaque"])
+def test_values_outside_the_packed_search(kind, k, prec):
+    # one odd record, a piece by itself, and plain ones behind it, whose supersegments are as the direct sweep gives them
+    import paper_2206_14503_gb300 as vdi
+
+    rng = np.random.default_rng(len(kind) + k)
+    pixels = []
+    for p in range(40):
+        lists = [_sorted(rng, 5) for _ in range(k)]
+        for r in lists:
+            r[:, :2] += 2.0  # behind the odd record, whose depths are 0 to 1
+        if p % 3 == 1:
+            rec = np.array([[0.0, 1.0, 0.25, 0.5, 0.125, 0.5]])
+            if kind == "short behind opaque":
+                # 1e-36 of the opaque record's length
+                rec = np.array([[-1.0, 0.0, 0.25, 0.5, 0.125, 1.0], [0.0, 1e-36, 0.5, 0.0, 0.125, 0.5]])
+            else:
+                at, v = ODD[kind]
+                rec[0, at] = v
+            if kind == "back far":  # the last of its list
+                rec[0, 0] = 10.0
+            e = p % k
+            lists[e] = np.concatenate([lists[e], rec] if kind == "back far" else [rec, lists[e]])
+        pixels.append(lists)
+    with np.errstate(invalid="ignore", over="ignore", divide="ignore"):
+        lists = [_compact(pixels, e) for e in range(k)]
+        _same(lists, prec, 3, 2, (vdi.VDI_SCHED_STAGED,) + ((1, vdi.VDI_SCHED_LANE) if k <= 8 else ()))
