@@ -1395,6 +1395,7 @@ __device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem<RMAX>& 
                 const float4 term = r < R ? S.term[r] : make_float4(0.f, 0.f, 0.f, 0.f);
                 const bool valid = fb.y > fb.x;
                 const unsigned m = __ballot_sync(0xffffffffu, valid);
+                __syncwarp();  // every lane has read its slot (a ballot orders no memory)
                 if (valid) {
                     const uint32_t c = n + __popc(m & ((1u << lane) - 1u));
                     S.rfb[c] = fb;

@@ -99,3 +99,19 @@ def test_values_outside_the_packed_search(kind, k, prec):
     with np.errstate(invalid="ignore", over="ignore", divide="ignore"):
         lists = [_compact(pixels, e) for e in range(k)]
         _same(lists, prec, 3, 2, (vdi.VDI_SCHED_STAGED,) + ((1, vdi.VDI_SCHED_LANE) if k <= 8 else ()))
+
+
+@pytest.mark.parametrize("n", [3, 26, 33, 93])
+@pytest.mark.parametrize("full", [0.1, 0.9])
+def test_records_without_length(n, full):
+    # the pooled builds (one warp up to 288 records a pixel, four above) move the others forward over the empty ones
+    import paper_2206_14503_gb300 as vdi
+
+    rng = np.random.default_rng(n)
+    k, pixels = 11, []
+    for p in range(45):
+        lists = [_sorted(rng, n) for _ in range(k)]
+        for r in lists:
+            r[rng.random(n) > full, 1] = 0.0
+        pixels.append(lists)
+    _same([_compact(pixels, e) for e in range(k)], 0, 5, 2, (vdi.VDI_SCHED_STAGED,))
