@@ -421,7 +421,10 @@ size_t vdi_batch_table_bytes(const vdi_request* reqs, int32_t n);
  * passed to vdi_composite_batched.  All requests must share one input
  * precision. */
 vdi_status vdi_batch_table_pack(const vdi_request* reqs, int32_t n, void* host_table, size_t bytes);
-/* Workspace bytes for a packed table (host_table from vdi_batch_table_pack). */
+/* Workspace bytes for a packed table (host_table from vdi_batch_table_pack):
+ * its pool holds the pieces of input lists of up to out.n_s records.  Where
+ * lists are longer, a pixel takes the room that its pieces need, and pixels
+ * for which none is left take the direct sweep. */
 size_t vdi_composite_batched_workspace(const void* host_table);
 /* Composites every request of the table with the pooled schedule run over all
  * of them at once: a persistent build launch in which warps take (request,

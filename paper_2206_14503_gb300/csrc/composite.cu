@@ -406,6 +406,17 @@ __device__ __forceinline__ unsigned long long* pool_used(uint32_t* list) {
     return reinterpret_cast<unsigned long long*>(list + 2);
 }
 
+// Takes `need` slots of a pool of `cap`, if it has them.  One that plainly does not fit takes nothing, so that smaller
+// ones still do; one that others overtake at the pool's end is lost.  (Taking nothing in that case either, by compare
+// and swap, costs a retry for every taker in between: the build of 640 x 480 pixels, K = 9, N_S = 4 took 2.5 times as
+// long.)
+__device__ __forceinline__ bool pool_take(unsigned long long* used, uint32_t need, uint32_t cap, uint32_t& at) {
+    if (*reinterpret_cast<volatile unsigned long long*>(used) + need > cap) return false;
+    const unsigned long long first = atomicAdd(used, (unsigned long long)need);
+    at = (uint32_t)first;
+    return first + need <= cap;
+}
+
 // slots of a pixel's run of n pieces in the pool (the search reads four pieces at once)
 __device__ __forceinline__ uint32_t run_slots(uint32_t n) { return (n + 3u) & ~3u; }
 
@@ -1092,6 +1103,7 @@ __device__ __forceinline__ void finish_pixel(const OutDev& out, uint32_t p, int 
 constexpr int kStageRMax = 1024;   // records per pixel held by the largest stage
 constexpr int kStageRSmall = 288;  // records per pixel of a batch that single warps build
 constexpr int kStageWarps = 4;     // warps per CTA, of either kind
+constexpr uint64_t kPoolPiecesPerPixel = 2 * kStageRMax;  // pieces that a pixel may need
 
 #ifndef VDI_BUILD_MIN_BLOCKS
 #define VDI_BUILD_MIN_BLOCKS 5
@@ -1231,27 +1243,26 @@ __device__ __forceinline__ void stage_walk(const StageSmem<RMAX>& S, const uint1
     }
 }
 
-// Where phase G writes a pixel's pieces: column `col` of its batch's part of the pool, rows of 4 pieces by
-// `ncol` columns.  A lane of the search then reads whole sectors, and the lanes that search a batch's pixels
-// together read neighbouring ones.  (One run per pixel, allocated as it was built, put the runs of a batch 60 MB
-// apart: every lane of the search in pages of its own.)
+// Where phase G writes a pixel's pieces: a column of its batch's part of the pool, rows of 4 pieces by `ncol`
+// columns.  A lane of the search then reads whole sectors, and the lanes that search a batch's pixels together read
+// neighbouring ones.  (One run per pixel, allocated as it was built, put the runs of a batch 60 MB apart: every lane
+// of the search in pages of its own.)  A run of its own is a column of one (build_batch says when).
 struct PoolColumn {
-    float4* A;  // of the batch's first piece
-    float2* B;
-    int col, ncol;
+    uint32_t base;  // slot of the first piece
+    int ncol;
     __device__ __forceinline__ size_t at(uint32_t row) const {
-        return ((size_t)(row >> 2) * ncol + col) * 4 + (row & 3);
+        return (size_t)base + (size_t)(row >> 2) * ncol * 4 + (row & 3);
     }
 };
 
 // Phase G after the merge: exact prefix scan of the records' terms over the
 // sorted bounds (srt, E of them; nv valid records), in contiguous chunks per
-// thread, and the pieces written to the column.  tot: scratch for the warps' totals.
-// Returns false when a piece is not packable.
-template <int NW, int PREC, bool OPQ, int RMAX>
+// thread, and the pieces written to the column that place(number of pieces, column) gives.  tot: scratch for the
+// warps' totals.  Returns false when it gives none or a piece is not packable.
+template <int NW, int PREC, bool OPQ, int RMAX, typename PLACE>
 __device__ __forceinline__ bool stage_scan(const PeIn* pe, StageSmem<RMAX>& S, ScanState* tot, const uint16_t* srt,
-                                           uint32_t E, uint32_t nv, const PoolColumn& out, int& npieces, int& nt,
-                                           float& f0) {
+                                           uint32_t E, uint32_t nv, const PiecePool& pool, const PLACE& place,
+                                           PoolColumn& out, int& npieces, int& nt, float& f0) {
     constexpr uint32_t T = 32 * NW;
     const int lane = threadIdx.x & 31, rank = group_rank<NW>();
     const uint32_t chunk = ((E + T - 1) / T) | 1u;  // (odd: the threads' reads of their chunks spread over the banks)
@@ -1291,6 +1302,7 @@ __device__ __forceinline__ bool stage_scan(const PeIn* pe, StageSmem<RMAX>& S, S
             }
         }
     }
+    if (!place(total_pieces, out)) return false;
     // the pieces: after bound i the active set is that of [key_i, key_{i+1}]
     uint32_t my_nt = 0;  // non-transparent pieces; from bit 16 on: pieces that are not packable
     uint32_t row = st.nb;
@@ -1312,8 +1324,8 @@ __device__ __forceinline__ bool stage_scan(const PeIn* pe, StageSmem<RMAX>& S, S
         Piece x;
         piece_from<true>(st.s, whole, wc, t, t1, x);
         const size_t at = out.at(row);
-        out.A[at] = make_float4(x.P[0], x.P[1], x.P[2], x.a);
-        out.B[at] = make_float2(x.b, x.lgT);
+        pool.A[at] = make_float4(x.P[0], x.P[1], x.P[2], x.a);
+        pool.B[at] = make_float2(x.b, x.lgT);
         my_nt += (x.a > 0.f ? 1u : 0u) + (packable(x) ? 0u : 1u << 16);
         ++row;
     });
@@ -1329,11 +1341,12 @@ __device__ __forceinline__ bool stage_scan(const PeIn* pe, StageSmem<RMAX>& S, S
     return my_nt < 1u << 16;
 }
 
-// Phase G for pixel p (at most RMAX records) by NW warps.  Returns false when a list is out of depth order or a piece
-// is not packable.
-template <int NW, int PREC, int RMAX>
-__device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem<RMAX>& S, ScanState* tot,
-                            const PoolColumn& out, int& npieces, int& nt, float& f0) {
+// Phase G for pixel p (at most RMAX records) by NW warps, its pieces to the column `out` of place.  Returns false when
+// a list is out of depth order, a piece is not packable or place gives no column.
+template <int NW, int PREC, int RMAX, typename PLACE>
+__device__ __forceinline__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem<RMAX>& S, ScanState* tot,
+                                            const PiecePool& pool, const PLACE& place, PoolColumn& out, int& npieces,
+                                            int& nt, float& f0) {
     constexpr uint32_t T = 32 * NW;
     const int lane = threadIdx.x & 31;
     const uint32_t rank = (uint32_t)group_rank<NW>();
@@ -1486,15 +1499,19 @@ __device__ bool stage_pixel(const PeIn* pe, int k, uint32_t p, StageSmem<RMAX>& 
         group_sync<NW>();
     }
     const uint16_t* srt = S.pay[src];
-    const bool ok = opaque ? stage_scan<NW, PREC, true>(pe, S, tot, srt, E, nv, out, npieces, nt, f0)
-                           : stage_scan<NW, PREC, false>(pe, S, tot, srt, E, nv, out, npieces, nt, f0);
+    const bool ok = opaque ? stage_scan<NW, PREC, true>(pe, S, tot, srt, E, nv, pool, place, out, npieces, nt, f0)
+                           : stage_scan<NW, PREC, false>(pe, S, tot, srt, E, nv, pool, place, out, npieces, nt, f0);
     group_sync<NW>();
     return ok;
 }
 
 // One batch of 32 pixels (from p0 on, at most p1) of a request: if its longest pixel is this kernel's (more than
-// RMIN and at most RMAX records, or beyond every stage), allocates the batch's columns of the pool at once (its
-// longest pixel's bound for each) and builds them pixel by pixel.  emit(pixel, entry) is called by the lane of
+// RMIN and at most RMAX records, or beyond every stage), takes columns of the pool for the batch (its longest pixel's
+// bound for each) and builds the pixels one by one.  RUNS: the pool is not sized for the worst case but for
+// `share` slots a pixel, and a batch whose columns would be longer takes a run for each pixel instead, of the slots
+// that its pieces need; so does a batch that the pool has no columns for.  (One pixel of 960 records among 31 of 64
+// took 32 columns of 1920, and most of the other batches went to the direct sweep: 256 x 256, K = 16, 62 ms, with
+// runs 8.1.)  emit(pixel, entry) is called by the lane of
 // warp 0 that has the pixel, for pixels with pieces and for those left to the direct sweep (the pixel's top bit);
 // pixels without records are finished here.
 struct BatchPixel {
@@ -1503,10 +1520,11 @@ struct BatchPixel {
     float f0;
 };
 
-template <int NW, int PREC, int RMIN, int RMAX>
+template <int NW, int PREC, int RMIN, int RMAX, bool RUNS>
 __device__ __forceinline__ bool build_batch(const PeIn* pe, int k, uint32_t p0, uint32_t p1, const OutDev& out,
-                                            const PiecePool& pool, unsigned long long* used,
-                                            StageSmem<RMAX>& S, ScanState* tot, unsigned long long* share, BatchPixel& mine) {
+                                            const PiecePool& pool, unsigned long long* used, uint32_t share,
+                                            StageSmem<RMAX>& S, ScanState* tot, uint32_t* base_of_all,
+                                            BatchPixel& mine) {
     const int lane = threadIdx.x & 31;
     const int ncol = (int)min(32u, p1 - p0);
     // (every warp of the group sums the counts for itself)
@@ -1516,37 +1534,51 @@ __device__ __forceinline__ bool build_batch(const PeIn* pe, int k, uint32_t p0, 
     const uint32_t fit = R <= (uint32_t)kStageRMax ? R : 0u;
     const uint32_t longest = __reduce_max_sync(0xffffffffu, fit);
     if (longest > (uint32_t)RMAX || (RMIN > 0 && longest <= (uint32_t)RMIN)) return false;
-    unsigned long long at = 0;
-    bool room = true;
-    if (longest > 0) {
-        const uint32_t need = run_slots(2 * longest - 1) * (uint32_t)ncol;
-        if (group_rank<NW>() == 0) at = atomicAdd(used, (unsigned long long)need);
+    // slots for every thread of the group, kNoSlots where the pool has not that many
+    constexpr uint32_t kNoSlots = 0xFFFFFFFFu;
+    auto take = [&](uint32_t need) {
+        uint32_t at = kNoSlots;
+        if (group_rank<NW>() == 0 && !pool_take(used, need, pool.cap, at)) at = kNoSlots;
         if constexpr (NW == 1) {
             at = __shfl_sync(0xffffffffu, at, 0);
         } else {
-            if (threadIdx.x == 0) *share = at;
+            if (threadIdx.x == 0) *base_of_all = at;
             __syncthreads();
-            at = *share;
+            at = *base_of_all;
         }
-        room = at + need <= (unsigned long long)pool.cap;
+        return at;
+    };
+    uint32_t base = kNoSlots;
+    if (longest > 0) {
+        const uint32_t rows = run_slots(2 * longest - 1);
+        if (!RUNS || rows <= share) base = take(rows * (uint32_t)ncol);
     }
-    const uint32_t base = room ? (uint32_t)at : 0u;
     mine.have = false;
     for (int col = 0; col < ncol; ++col) {
         const uint32_t p = p0 + (uint32_t)col;
         const uint32_t n_rec = __shfl_sync(0xffffffffu, R, col);
         int n = 0, nt = 0;
         float f0 = 0.f;
-        bool ok = n_rec <= (uint32_t)kStageRMax && room;
+        bool ok = n_rec <= (uint32_t)kStageRMax;
+        PoolColumn at{0u, 1};
+        auto place = [&](uint32_t n_pieces, PoolColumn& c) {
+            if (!RUNS || base != kNoSlots) {
+                c = PoolColumn{base + (uint32_t)col * 4u, ncol};
+            } else {
+                group_sync<NW>();  // the last run's first slot has been read
+                c = PoolColumn{take(run_slots(n_pieces)), 1};
+            }
+            return RUNS ? c.base != kNoSlots : true;
+        };
         if (ok && n_rec > 0)
-            ok = stage_pixel<NW, PREC>(pe, k, p, S, tot, PoolColumn{pool.A + base, pool.B + base, col, ncol}, n, nt, f0);
+            ok = (RUNS || base != kNoSlots) && stage_pixel<NW, PREC>(pe, k, p, S, tot, pool, place, at, n, nt, f0);
         if (lane == col) {
             if (!ok) {
                 mine = BatchPixel{true, p | 0x80000000u, 0u, 0u, 0.f};
             } else if (n == 0) {
                 if (NW == 1 || threadIdx.x < 32) finish_pixel(out, p, 0, 0.f);  // no record: an empty list
             } else {
-                mine = BatchPixel{true, p, base + (uint32_t)col * 4u, pack_pieces((uint32_t)n, (uint32_t)nt, ncol), f0};
+                mine = BatchPixel{true, p, at.base, pack_pieces((uint32_t)n, (uint32_t)nt, at.ncol), f0};
             }
         }
     }
@@ -2150,8 +2182,7 @@ template <int NW, int RMAX>
 struct BuildShared {
     StageSmem<RMAX> stage[NW == 1 ? kStageWarps : 1];
     ScanState tot[NW == 1 ? 1 : NW];
-    unsigned long long base;
-    uint32_t item;
+    uint32_t base, item;
     __device__ BuildShared() {}
 };
 
@@ -2178,8 +2209,9 @@ __global__ void __launch_bounds__(kStageWarps * 32, VDI_BUILD_MIN_BLOCKS) compos
         const uint32_t batch = next_item<NW>(ba.counter + (NW == 1 ? 0 : 1), &sh.item);
         if (batch >= nbatch) break;
         BatchPixel px;
-        if (!build_batch<NW, PREC, RMIN, RMAX>(a.pe, a.k, ba.p0 + batch * 32u, ba.p1, a.out, ba.pool, pool_used(ba.list),
-                                               sh.stage[NW == 1 ? threadIdx.x >> 5 : 0], sh.tot, &sh.base, px))
+        if (!build_batch<NW, PREC, RMIN, RMAX, false>(a.pe, a.k, ba.p0 + batch * 32u, ba.p1, a.out, ba.pool,
+                                                      pool_used(ba.list), 0u, sh.stage[NW == 1 ? threadIdx.x >> 5 : 0],
+                                                      sh.tot, &sh.base, px))
             continue;
         if (NW > 1 && threadIdx.x >= 32) continue;
         list_push(ba.list, px.have, FlatEntry{px.p, px.base, px.n_nt, px.f0});
@@ -2667,6 +2699,14 @@ struct BatchEntry {
     uint32_t req, pad0, pad1, pad2;
 };
 
+// Pieces that a request's pixel is expected to need: its K lists of at most N_S records cut into at most
+// 2 K N_S - 1 pieces, rounded up to the groups of four that a run takes, at most the stage's.  (Lists may be longer:
+// the table does not say by how much.)
+__host__ __device__ static uint64_t batch_pixel_pieces(const ReqDev& r) {
+    const uint64_t est = (2ull * (uint64_t)r.k * (uint64_t)(r.out.n_s > 0 ? r.out.n_s : 1) + 2) / 4 * 4;
+    return est < kPoolPiecesPerPixel ? est : kPoolPiecesPerPixel;
+}
+
 struct BatchBuildArgs {
     unsigned int* counter;  // item counter
     uint32_t* list;         // [0] entries, [1] next entry of the flat pass, [2], [3] pool pieces taken; entries from word 8
@@ -2698,8 +2738,9 @@ __global__ void __launch_bounds__(kStageWarps * 32, VDI_BUILD_MIN_BLOCKS) compos
         const uint32_t base = (item - r.item_begin) * 32u;
         BatchPixel px;
         if (r.schedule == VDI_SCHED_STAGED) {
-            if (!build_batch<NW, PREC, RMIN, RMAX>(a.pes + r.pe_begin, r.k, base, r.npix, r.out, bb.pool, pool_used(bb.list),
-                                                   sh.stage[NW == 1 ? threadIdx.x >> 5 : 0], sh.tot, &sh.base, px))
+            if (!build_batch<NW, PREC, RMIN, RMAX, true>(a.pes + r.pe_begin, r.k, base, r.npix, r.out, bb.pool,
+                                                         pool_used(bb.list), (uint32_t)batch_pixel_pieces(r),
+                                                         sh.stage[NW == 1 ? threadIdx.x >> 5 : 0], sh.tot, &sh.base, px))
                 continue;
             if (NW > 1 && threadIdx.x >= 32) continue;
         } else {
@@ -2741,15 +2782,33 @@ template <int P, int PREC>
 __global__ void __launch_bounds__(128) composite_batched_marked_kernel(const __grid_constant__ BatchArgs a,
                                                                        const uint32_t* __restrict__ list) {
     extern __shared__ uint32_t smem[];
+    // a warp collects the marked entries among the others until it has one for every lane (where the pool runs out
+    // within batches, a quarter of the entries are marked: 256 x 256, K = 16, lists 1.4 N_S long, 16.4 -> 11.3 ms)
+    __shared__ uint32_t queue[4][64];
+    uint32_t* q = queue[threadIdx.x >> 5];
     const uint32_t n = *list;
     const BatchEntry* entries = reinterpret_cast<const BatchEntry*>(list + 8);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i - threadIdx.x < n; i += gridDim.x * blockDim.x) {
-        const BatchEntry en = i < n ? entries[i] : BatchEntry{0u, 0u, 0u, 0.f, 0u, 0u, 0u, 0u};
-        if (en.p & 0x80000000u) {
+    const uint32_t lane = threadIdx.x & 31, warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+    uint32_t queued = 0;
+    for (uint32_t i0 = warp * 32; i0 < n || queued > 0; i0 += warps * 32) {
+        const bool more = i0 < n, marked = more && i0 + lane < n && (entries[i0 + lane].p & 0x80000000u);
+        const unsigned m = __ballot_sync(0xffffffffu, marked);
+        if (marked) q[queued + __popc(m & ((1u << lane) - 1u))] = i0 + lane;
+        queued += __popc(m);
+        __syncwarp();
+        if (more && queued < 32) continue;
+        if (lane < queued) {
+            const BatchEntry en = entries[q[lane]];
             const ReqDev& r = a.reqs[en.req];
             composite_pixel<0, P, 2, PREC>(a.pes + r.pe_begin, r.k, r.out, a.iters, a.status, en.p & 0x7FFFFFFFu,
                                            smem);
         }
+        const uint32_t rest = queued > 32 ? queued - 32 : 0u;
+        const uint32_t next = lane < rest ? q[32 + lane] : 0u;
+        __syncwarp();
+        if (lane < rest) q[lane] = next;
+        queued = rest;
     }
 }
 
@@ -2875,9 +2934,6 @@ static cudaError_t launch_flat(bool census, const CompArgs& a, const PiecePool& 
     k2<<<(unsigned)b, 128, 0, st>>>(a, pool, list);
     return cudaGetLastError();
 }
-
-// pieces a pixel of the pooled staged path may need (the stage holds kStageRMax records)
-constexpr uint64_t kPoolPiecesPerPixel = 2 * kStageRMax;
 
 template <int PREC>
 static cudaError_t launch_staged_pool(bool census, const CompArgs& a, void* workspace, size_t ws_bytes,
@@ -3066,17 +3122,9 @@ vdi_status batch_table_pack(const vdi_request* reqs, int n, void* host_table, si
     return VDI_OK;
 }
 
-// Pooled batched path: pieces a request's pixel is expected to need (its K lists of at most N_S records
-// cut into at most 2 K N_S - 1 pieces, at most the stage's), and the workspace: [header][counter]
-// [list: 8 words, kBatchListCap entries at most][pool]
+// Pooled batched path, its workspace: [header][counter][list: 8 words, kBatchListCap entries at most][pool]
 constexpr uint64_t kBatchListCap = 1u << 22;
 constexpr uint64_t kBatchPoolCap = 1u << 28;
-
-static uint64_t batch_pixel_pieces(const ReqDev& r) {
-    // (rounded up to the groups of four that a run takes)
-    const uint64_t est = (2ull * (uint64_t)r.k * (uint64_t)(r.out.n_s > 0 ? r.out.n_s : 1) + 2) / 4 * 4;
-    return est < kPoolPiecesPerPixel ? est : kPoolPiecesPerPixel;
-}
 
 static size_t batch_list_bytes(const BatchHeader* hd) {
     const uint64_t n = hd->total_pixels < kBatchListCap ? hd->total_pixels : kBatchListCap;
