@@ -498,7 +498,8 @@ vdi_status vdi_mlp_infer(const void* model, const float* feats, int32_t n, float
  * of the prediction over the rows with valid != 0.  vdi_mlp_grad writes the
  * gradient (device float[6849]) and the loss (device float); vdi_mlp_train_step
  * also applies one Adam step (beta 0.9, 0.999, eps 1e-8, learning rate lr).
- * Deterministic (per-block partial sums in the workspace, fixed-order reduction). */
+ * Deterministic, and the same on every device (a fixed number of partial sums in
+ * the workspace, reduced in a fixed order). */
 size_t vdi_mlp_train_workspace(int32_t n);
 vdi_status vdi_mlp_grad(const void* model, const float* feats, const float* labels, const uint8_t* valid, int32_t n,
                         float* grad, float* loss, void* workspace, size_t ws_bytes, vdi_stream stream);

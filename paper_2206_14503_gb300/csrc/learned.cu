@@ -720,30 +720,25 @@ vdi_status launch_gamma_expand(float* const* gammas, int k, int w, int h, const 
     return cuda_check(cudaGetLastError(), "gamma_expand_kernel launch");
 }
 
+// (Room for a partial gradient per tile and one more, as programs have it from before the passes took at most
+// kTrainCtas: a size that was refused stays refused.)
 size_t train_workspace(int n) {
     size_t blocks = ((size_t)n + kTrainRows - 1) / kTrainRows;
     return 256 + align_up(blocks * (kNP + 1) * sizeof(float), 256) + align_up((kNP + 1) * sizeof(float), 256);
 }
 
-// Two CTAs per SM hold their tiles (106 KB each); a CTA takes several tiles, so that few partial gradients are
-// written and summed.
-static vdi_status train_blocks(int n, int& blocks) {
-    int dev = 0, sms = 0;
-    vdi_status s = cuda_check(cudaGetDevice(&dev), "cudaGetDevice");
-    if (s == VDI_OK) s = cuda_check(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-    const int tiles = (n + kTrainRows - 1) / kTrainRows;
-    blocks = tiles < 2 * sms ? tiles : 2 * sms;
-    return s;
-}
+// CTAs of a training pass, each of several tiles, so that few partial gradients are written and summed: two for each
+// of the 152 SMs, as many as their tiles (106 KB each) allow.  A constant and not the device's count, so that the
+// order of the sums, and with it a step's bits, is the same on every device.
+constexpr int kTrainCtas = 304;
 
 template <bool STEP>
 static vdi_status launch_train(unsigned char* model, const float* x, const float* y, const unsigned char* valid, int n,
                                float* grad, float lr, float* loss, void* ws, cudaStream_t st) {
-    int blocks = 0;
-    vdi_status s = train_blocks(n, blocks);
-    if (s != VDI_OK || blocks == 0) return s;
+    const int tiles = (n + kTrainRows - 1) / kTrainRows, blocks = tiles < kTrainCtas ? tiles : kTrainCtas;
+    if (blocks == 0) return VDI_OK;
     float* partial = reinterpret_cast<float*>(static_cast<char*>(ws) + 256);
-    s = cuda_check(cudaFuncSetAttribute(mlp_fwdbwd_kernel<STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    vdi_status s = cuda_check(cudaFuncSetAttribute(mlp_fwdbwd_kernel<STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)sizeof(TrainSmem)),
                    "smem attribute");
     if (s != VDI_OK) return s;
