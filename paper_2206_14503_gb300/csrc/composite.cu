@@ -1048,7 +1048,7 @@ struct FlatEntry {
 
 // n and nt below 2048 (a stage of 1024 records has at most 2047 pieces, a lane's slab of 480 at most 959), 32 columns
 __device__ __forceinline__ uint32_t pieces_of(uint32_t n_nt) { return n_nt & 0x7FFu; }
-__device__ __forceinline__ uint32_t opaque_of(uint32_t n_nt) { return n_nt >> 11 & 0x7FFu; }
+__device__ __forceinline__ uint32_t nontransparent_of(uint32_t n_nt) { return n_nt >> 11 & 0x7FFu; }
 __device__ __forceinline__ uint32_t columns_of(uint32_t n_nt) { return (n_nt >> 22) + 1u; }
 __device__ __forceinline__ uint32_t pack_pieces(uint32_t n, uint32_t nt, int ncol) {
     return n | nt << 11 | (uint32_t)(ncol - 1) << 22;
@@ -1084,22 +1084,21 @@ __device__ __forceinline__ void finish_pixel(const OutDev& out, uint32_t p, int 
 // ---------------------------------------------------------------------------
 // Staged path
 // ---------------------------------------------------------------------------
-// A warp (or a CTA of four, for long lists) takes 32 consecutive pixels at a time.  Phase G builds the pieces of
-// each of them in turn, every thread on one pixel: they load the pixel's
-// records from all K lists, drops those with b <= f, sorts their bounds (each
-// list's bounds are already in order, so a stable merge of the K runs: log2 K
-// rounds in which every bound finds its place in its partner run by binary
-// search; ties go to the lower PE) and obtains the active set's sums after
-// every bound by an exact prefix scan of the records' terms.  The pieces go to
-// the warp's piece buffer, pixel i of the batch in column i.  Phase S: lane i
-// runs the search and the emission of pixel i over column i.  The pieces are
-// bit for bit those of the direct sweep.  Pixels with more records than the
-// stage holds are listed for the direct path (a second launch).
+// A warp (or a CTA of four, for long lists) takes 32 consecutive pixels at a time and builds the pieces of each of
+// them in turn, every thread on one pixel: they load the pixel's records from all K lists, drop those with b <= f,
+// sort their bounds (each list's bounds are already in order, so a stable merge of the K runs: log2 K rounds in which
+// every bound finds its place in its partner run by binary search; ties go to the lower PE) and obtain the active
+// set's sums after every bound by an exact prefix scan of the records' terms.  The pieces go to the pixel's column of
+// the pool, and the pixel to the list of the flat search (a later launch).  They are bit for bit those of the direct
+// sweep, which takes the pixels that this path cannot (the file's header lists them).
 
-// A pixel is built by one warp when its 32-pixel batch's lists are short, by a CTA of four when they are long:
-// the steps are chains of dependent shared-memory reads, so what counts is the warps an SM holds.  A warp's
-// stage of 1024 records (20 KB, a 172 KB CTA of 8 warps) left 8 warps per SM, 17% of the issue slots used; four
-// warps on such a stage make 40, and short lists take a stage of 288 records (11 KB) each.
+// A pixel is built by one warp when its 32-pixel batch's lists are short, by a CTA of four when they are long: the
+// steps are chains of dependent shared-memory reads, so what counts is the warps an SM holds.  A warp's stage of 1024
+// records (20 KB, a 172 KB CTA of 8 warps) left 8 warps per SM, 17% of the issue slots used; four warps on such a
+// stage (38 KB with the records' terms, five CTAs) make 20, and a stage of 288 records for each warp (46 KB a CTA,
+// four CTAs) 16 without barriers.  The line lies where the two are equal: 131,072 pixels, K = 12, dense, of 144
+// records one warp takes 4.53 ms and four 5.02, of 240 7.09 and 7.36, of 276 8.22 and 8.25, of 288 8.65 and 8.55.
+// (A stage of 284 records lets a fifth CTA in: 4.51, 7.19, 8.17 ms.)
 constexpr int kStageRMax = 1024;   // records per pixel held by the largest stage
 constexpr int kStageRSmall = 288;  // records per pixel of a batch that single warps build
 constexpr int kStageWarps = 4;     // warps per CTA, of either kind
@@ -2162,13 +2161,11 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 4) composite_lane_kernel(cons
 }
 
 // ---------------------------------------------------------------------------
-// Pooled staged path (K > kLaneKMax): composite_build_kernel builds each
-// pixel's pieces as phase G of the staged schedule does -- the whole warp on
-// one pixel: coalesced span loads, a stable merge of the bounds, the exact
-// prefix scan of the mixture terms -- but writes them as one run of the pool
-// and lists the pixel; composite_flat_kernel then searches and emits every
-// listed pixel, a lane each.  The host runs the pixels in chunks whose pieces
-// fit the pool.
+// Pooled staged path (K > kLaneKMax): two launches of composite_build_kernel
+// (build_batch's warps and CTAs of four) build the pixels' pieces into their
+// batches' columns of the pool and list the pixels; composite_flat_kernel then
+// searches and emits every listed pixel, a lane each.  The host runs the pixels
+// in chunks whose pieces fit the pool.
 // ---------------------------------------------------------------------------
 struct BuildArgs {
     unsigned int* counter;  // batch counter
@@ -2231,8 +2228,9 @@ __global__ void __launch_bounds__(kStageWarps * 32, VDI_BUILD_MIN_BLOCKS) compos
 // that finishes its pixel takes the next one from the list.  The decisions
 // are those of composite_search_emit, step for step, and the bisection is
 // replayed from the marches' counts (vdi_search.cuh), so the output is the
-// same, bit for bit.  The pieces come from a pool in the workspace (written by
-// the batch pass), one contiguous run per pixel.
+// same, bit for bit.  The pieces come from a pool in the workspace: a pixel's
+// column of its batch's rows (the pooled builds), or a run of its own, which is
+// a column of one (the lane path).
 //
 // What bounds it: instructions per piece (640 x 480, K = 32 dense: the search pass's two chunks of 131,072 pixels
 // took 35 ms each with three candidates value by value and a load per piece; the whole call 171 -> 70 ms with the
@@ -2351,7 +2349,7 @@ struct FlatSrcOne {
         L.p = en.p;
         L.base = en.base;
         L.n = (int)pieces_of(en.n_nt);
-        L.nt = (int)opaque_of(en.n_nt);
+        L.nt = (int)nontransparent_of(en.n_nt);
         L.ncol = (int)columns_of(en.n_nt);
         L.f0 = en.f0;
         L.out = out;
@@ -2503,13 +2501,13 @@ __device__ __forceinline__ void flat_loop(const SRC& src, const PiecePool& pool,
             const float4 A = S.A[j & 7][threadIdx.x];
             const float2 B = reinterpret_cast<const float2*>(&S.B[(j >> 1) & 3][threadIdx.x])[j & 1];
             const float b = B.x;
-            const bool opaque = A.w > 0.f;
+            const bool seen = A.w > 0.f;
             const PieceX x{{pk(A.x), pk(A.y), pk(A.z)},
                            pk(-A.w),
                            pk(fmaxf(B.y, -1e34f)),
                            pk(f),
                            pk(__fsub_rn(b, f)),
-                           pk(opaque ? 1.f : 0.f)};
+                           pk(seen ? 1.f : 0.f)};
             // one instruction stream for counting and emitting lanes: an emitting lane's first candidate carries
             // the budget and writes the supersegment a termination closes
             const f32x2 k = fp_keep(st[0], x, g2[0], last);
@@ -2521,7 +2519,7 @@ __device__ __forceinline__ void flat_loop(const SRC& src, const PiecePool& pool,
                     ++written;
                     last = written + 1 >= L.out->n_s;
                 }
-                bt = opaque ? b : bt;
+                bt = seen ? b : bt;
             }
             fp_apply(st[0], x, k);
 #pragma unroll
@@ -2687,9 +2685,9 @@ __device__ __forceinline__ int request_of(const BatchArgs& a, uint32_t item) {
 }
 
 // Pooled batched path: composite_batched_build_kernel takes (request,
-// 32-pixel batch) items of a chunk from an atomic counter and builds each
-// pixel's pieces into the pool as composite_build_kernel does (requests with
-// a direct schedule, and pixels the stage cannot hold, are listed for the
+// 32-pixel batch) items of a chunk from an atomic counter and builds the
+// pixels' pieces into the pool as composite_build_kernel does, into columns or
+// into runs (build_batch; requests with a direct schedule, and pixels the stage cannot hold, are listed for the
 // direct sweep); composite_batched_flat_kernel searches and emits the listed
 // pixels, a lane each, each into its request's output; composite_batched_
 // marked_kernel sweeps the pixels listed for the direct path.
@@ -2761,7 +2759,7 @@ struct FlatSrcBatch {
         L.p = en.p;
         L.base = en.base;
         L.n = (int)pieces_of(en.n_nt);
-        L.nt = (int)opaque_of(en.n_nt);
+        L.nt = (int)nontransparent_of(en.n_nt);
         L.ncol = (int)columns_of(en.n_nt);
         L.f0 = en.f0;
         L.out = &reqs[en.req].out;
@@ -2920,7 +2918,6 @@ static cudaError_t launch_marked(bool census, const CompArgs& a, const uint32_t*
     return cudaGetLastError();
 }
 
-template <int PREC>
 static cudaError_t launch_flat(bool census, const CompArgs& a, const PiecePool& pool, uint32_t* list, uint64_t lanes,
                                cudaStream_t st, int max_per_sm = 0) {
     auto k2 = census ? composite_flat_kernel<true> : composite_flat_kernel<false>;
@@ -2940,7 +2937,7 @@ static cudaError_t launch_staged_pool(bool census, const CompArgs& a, void* work
                                      cudaStream_t st) {
     // workspace: [header][counters][list: 4 words, entries of a chunk][pool: float4 x cap][pool: float2 x cap]
     // (the list stays in build order: dense pixels have equal piece counts, and a warp's lanes then read
-    // pool runs that one warp wrote next to each other)
+    // neighbouring columns of a batch)
     const uint64_t npix = (uint64_t)a.npix;
     char* base = static_cast<char*>(workspace);
     // the chunk: as many pixels as the pool holds at the stage's worst case, all of them if they fit
@@ -2970,7 +2967,7 @@ static cudaError_t launch_staged_pool(bool census, const CompArgs& a, void* work
         if (e != cudaSuccess) return e;
         e = launch_build<1, PREC>(census, a, ba, st);
         if (e == cudaSuccess) e = launch_build<kStageWarps, PREC>(census, a, ba, st);
-        if (e == cudaSuccess) e = launch_flat<PREC>(census, a, ba.pool, ba.list, p1 - p0, st, VDI_FLAT_CTAS_PER_SM);
+        if (e == cudaSuccess) e = launch_flat(census, a, ba.pool, ba.list, p1 - p0, st, VDI_FLAT_CTAS_PER_SM);
         if (e == cudaSuccess) {
             if (P == 16) e = launch_marked<0, 16, PREC>(census, a, ba.list, p1 - p0, st);
             else if (P == 32) e = launch_marked<0, 32, PREC>(census, a, ba.list, p1 - p0, st);
@@ -3020,7 +3017,7 @@ static cudaError_t launch_lane(bool census, const CompArgs& a, void* workspace, 
     // search pass over the list sorted by piece count: a persistent grid; the list's length is known
     // only on the device
     e = launch_sort<FlatEntry, 4>(la.list, sorted, hist, npix, st);
-    if (e == cudaSuccess) e = launch_flat<PREC>(census, a, la.pool, sorted, npix, st);
+    if (e == cudaSuccess) e = launch_flat(census, a, la.pool, sorted, npix, st);
     if (e != cudaSuccess) return e;
     return launch_marked<kLaneKMax, 16, PREC>(census, a, la.list, npix, st);
 }

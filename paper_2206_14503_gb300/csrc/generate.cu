@@ -574,24 +574,23 @@ __device__ __forceinline__ float bisect_gamma(const Ray& r, int k0, int k1, cons
     return ghi;
 }
 
+// samples on the way in the first march: the fixed-gamma kernel has the registers for two, the others do not (the
+// learned one with two: 0.94x to 1.11x of its time, by the host)
+#ifndef VDI_FIXED_AHEAD
+#define VDI_FIXED_AHEAD 2
+#endif
+
 // gamma and count of one (PE, ray): the body of the count kernels.  The
 // learned-gamma refinement (mode 3) is compiled only into the LEARNED
 // instantiation so that the search kernel keeps its register budget.  Every
 // march is inlined: out-of-line calls in this persistent loop cost far more
 // than the spills inlining brings (the learned choice took 80.6 ms with the
 // refinement, its marches and the search fallback out of line, 65.6 ms inlined).
-// samples on the way in the first march: the fixed-gamma kernel has the registers for two, the others do not
-#ifndef VDI_FIXED_AHEAD
-#define VDI_FIXED_AHEAD 2
-#endif
-#ifndef VDI_LEARNED_AHEAD
-#define VDI_LEARNED_AHEAD 1
-#endif
 template <bool LEARNED, bool OWNED, bool FIXED>
 __device__ __forceinline__ void count_ray(const GenReq& a, const BrickDev& b, const CompactDev& o, int e, int i, int j,
                                           const float4* __restrict__ lut2, const CacheRef& cref, Census& cs,
                                           unsigned long long& rays, uint2* rng) {
-    constexpr int kAhead = FIXED ? VDI_FIXED_AHEAD : (LEARNED ? VDI_LEARNED_AHEAD : 1);
+    constexpr int kAhead = FIXED ? VDI_FIXED_AHEAD : 1;
     const int mode = FIXED ? 0 : (LEARNED ? 3 : a.mode);
     const size_t p = (size_t)j * a.cam.W + i;
     Ray r;
@@ -722,8 +721,9 @@ __global__ void __launch_bounds__(kCountThreads, FIXED ? VDI_FIXED_MIN_BLOCKS
     if (CENSUS) census_flush_gen(cs, rays, a.status);
 }
 
-// samples on the way in the emission's march, and its block bound: 7 blocks hold two without spills (64^3 frame,
-// whose 200 samples a ray are one latency after the other: 300 -> 293 us)
+// samples on the way in the emission's march, and its block bound: 7 blocks hold two with little spilled (8 bytes
+// stored and 16 loaded a thread for box domains, 24 and 36 owned, 68 and 76 batched; 64^3 frame, whose 200 samples a
+// ray are one latency after the other: 300 -> 293 us)
 #ifndef VDI_EMIT_AHEAD
 #define VDI_EMIT_AHEAD 2
 #endif

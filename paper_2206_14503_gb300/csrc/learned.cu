@@ -358,7 +358,8 @@ __global__ void gamma_expand_kernel(const __grid_constant__ ExpandArgs a) {
 // deterministic on a device.
 //
 // The work is five products of 64-wide matrices per tile, 35 k operations a row
-// (0.03 ms for 65,536 rows at the FP32 rate), bound by FP32 issue when its
+// (0.029 ms for 65,536 rows at 80.5 TFLOP/s, an FMA a lane and clock counted as
+// two: 152 SMs of 128 lanes at 2070 MHz), bound by FP32 issue when its
 // operands come from shared memory in few wide reads: a thread computes 4 x 4
 // outputs, 16 FMAs for two 16-byte reads, and rows are padded to 68 (44) floats
 // so that the reads of a warp's row groups broadcast and its column groups fall

@@ -115,3 +115,15 @@ def test_records_without_length(n, full):
             r[rng.random(n) > full, 1] = 0.0
         pixels.append(lists)
     _same([_compact(pixels, e) for e in range(k)], 0, 5, 2, (vdi.VDI_SCHED_STAGED,))
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("total", [287, 288, 289, 1023, 1024, 1025])
+def test_stage_limits_of_many_lists(total, prec):
+    # K = 64 (every lane of the count's two loads), the longest pixel at the limits of one warp's stage and of four's
+    import paper_2206_14503_gb300 as vdi
+
+    rng = np.random.default_rng(total)
+    k = 64
+    pixels = [[_sorted(rng, (total + k - 1 - e) // k if p in (3, 40) else (p + e) % 3) for e in range(k)] for p in range(44)]
+    _same([_compact(pixels, e) for e in range(k)], prec, 7, 2, (vdi.VDI_SCHED_STAGED,))
